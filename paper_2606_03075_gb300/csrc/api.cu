@@ -526,7 +526,8 @@ int tgvkv_prefill(const tgvkv_desc* desc, const uint16_t* q, const uint16_t* k, 
     REQUIRE_PTR(workspace, "workspace", true);
     const WsLayout lay = layout_of(p);
     cudaError_t e = launch_prefill(p, q, k, v, modality, text_pos, o, q_text, row_stats,
-                                   status_of(workspace, lay), static_cast<cudaStream_t>(stream));
+                                   static_cast<char*>(workspace), lay,
+                                   static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? ok() : cuda_fail(e, "prefill launch");
 }
 

@@ -78,11 +78,13 @@ int score_launches(const Problem& p);
 int select_compact_launches(const Problem& p);
 
 // Causal prefill attention over every token (prefill.cu), which also writes
-// the eviction step's query rows (q_text) and their (m, Z, vision mass).
+// the eviction step's query rows (q_text) and their (m, Z, vision mass).  The
+// work counters in the workspace must be zero on entry; the kernel leaves them
+// zero.
 cudaError_t launch_prefill(const Problem& p, const uint16_t* q, const uint16_t* k,
                            const uint16_t* v, const uint8_t* modality, const int32_t* text_pos,
-                           uint16_t* o, uint16_t* q_text, float* row_stats, uint32_t* status,
-                           cudaStream_t stream);
+                           uint16_t* o, uint16_t* q_text, float* row_stats, char* ws,
+                           const WsLayout& lay, cudaStream_t stream);
 
 // TMA map of a bf16 [rows][d] tensor with boxes of 64 x box_rows, 128-byte
 // swizzle (score_tc.cu), and the SM count of the current device.

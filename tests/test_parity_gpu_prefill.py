@@ -423,3 +423,51 @@ def test_evict_with_statistics_head_budgets(api, stat):
     ko, vo = oracle.compact(inp["k"], inp["v"], off, idx)
     np.testing.assert_array_equal(g["k_out"], ko)
     np.testing.assert_array_equal(g["v_out"], vo)
+
+
+# head lengths at the edges of the kernel's work split: one tile, one pair of row
+# tiles, an odd tile left over, a last tile of one row; MHA and grouped heads.
+# "few" row tiles (one per item) and "many" (pairs of them, over three per SM).
+EDGES = [(1, 1, 64), (31, 4, 128), (128, 1, 128), (129, 2, 64), (256, 1, 64), (257, 3, 128),
+         (385, 1, 128), (513, 2, 128)]
+
+
+def _layers(form, heads, n):
+    return 2 if form == "few" else -(-600 // (heads * -(-n // 128)))
+
+
+@pytest.mark.parametrize("form", ["few", "many"])
+@pytest.mark.parametrize("n,group,d", EDGES)
+def test_prefill_tile_edges(api, n, group, d, form):
+    text = max(1, n // 5)
+    seg = [("text", 1)] if n == 1 else [("text", n - text - (n - text) // 2),
+                                        ("vision", (n - text) // 2), ("text", text)]
+    wl = synth.custom(f"edge{n}", _layers(form, 8 * group, n), 8 * group, 8, d,
+                      [s for s in seg if s[1] > 0], window="all_text")
+    inp = synth.generate_prefill(wl, seed=11)
+    out = _run_prefill(api, wl, inp)
+    _check_prefill(wl, inp, *out, layers=sorted({0, wl.L // 2, wl.L - 1}))
+
+
+@pytest.mark.parametrize("form", ["few", "many"])
+@pytest.mark.parametrize("first_rise", [20, 70, 140, 200, 330])
+def test_prefill_rising_logits(api, first_rise, form):
+    """Logits that jump along the sequence, so that the rows' reference maximum moves
+    inside the first tile and in later ones (the output then holds products against
+    the old reference, which must be rescaled once they have all been added).  The
+    first 16 dimensions of the queries are positive and the keys' there rise in steps,
+    by about 3 and then 20 base-2 units per step."""
+    wl = synth.custom("rising", _layers(form, 8, 440), 8, 4, 64,
+                      [("text", 40), ("vision", 300), ("text", 100)], window="all_text")
+    inp = synth.generate_prefill(wl, seed=12)
+    q = oracle.widen_bf16(inp["q_all"]).astype(np.float32)
+    k = oracle.widen_bf16(inp["k"]).astype(np.float32)
+    q[..., :16] = 0.5 + np.abs(q[..., :16])
+    step = np.zeros(wl.N, np.float32)
+    step[first_rise:] = 1.5
+    step[first_rise + 45:] = 9.0
+    k[..., :16] = step[:, None] + 0.01 * k[..., :16]
+    inp["q_all"], inp["k"] = synth.to_bf16_bits(q), synth.to_bf16_bits(k)
+    inp["q"] = inp["q_all"][:, :, inp["text_pos"]]
+    out = _run_prefill(api, wl, inp)
+    _check_prefill(wl, inp, *out, layers=sorted({0, wl.L - 1}))
