@@ -102,10 +102,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
-__device__ __forceinline__ void fence_proxy_async() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 __device__ __forceinline__ int clampi(long long x, int lo, int hi) {
     return x < lo ? lo : (x > hi ? hi : (int)x);
 }
@@ -270,16 +266,11 @@ decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ C
             }
         }
     }
-    // Zero the rings once: the rows of a k-step that no box of a short chunk
-    // loads then hold zeros or rows of an earlier chunk, never stale bits.
-    for (int i = tid; i < Gm::kRing / 16; i += blockDim.x)
-        reinterpret_cast<uint4*>(ring)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) never = 0;
     if (lane == 0) {
         for (int st = 0; st < kDecStages; ++st) tc::mbar_init(&tl.full[warp][st], 1);
         tc::fence_mbar_init();
     }
-    fence_proxy_async();   // the zeroed rings before any TMA write to them
     __syncthreads();
 
     rows.R0 = rows.at(0);
@@ -409,7 +400,10 @@ decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ C
                                            pr[4 * kk + 1] - __uint_as_float(h01 & 0xFFFF0000u));
             const uint32_t l23 = pack_bf16(pr[4 * kk + 2] - __uint_as_float(h23 << 16),
                                            pr[4 * kk + 3] - __uint_as_float(h23 & 0xFFFF0000u));
-            const int row = 16 * kk + (lane & 7) + ((lane >> 3) & 1) * 8;
+            // keys that no box of a short chunk loaded: any loaded row stands in (P is 0
+            // there, and the stale bits of the ring must not meet it as a NaN)
+            int row = 16 * kk + (lane & 7) + ((lane >> 3) & 1) * 8;
+            if (row >= ((c.n + 7) & ~7)) row = lane & 7;
 #pragma unroll
             for (int nd2 = 0; nd2 < ND / 2; ++nd2) {
                 const int unit = 2 * nd2 + (lane >> 4);
@@ -477,96 +471,50 @@ decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ C
     }
 }
 
-// The split sets' merge, the CSR check and the empty sets: one warp per
-// (set, query head of the pass).  Launched as a programmatic dependent of
-// decode_kernel: it reads its inputs, then waits for that grid's partial
-// results.  A split set's partials are combined in stream order: the lanes
-// fetch the streams' (m, l) side by side, so the common maximum and every
-// weight cost one round trip; then lane t adds dims [t * D/32, (t+1) * D/32)
-// of the weighted O of each stream, loading 8 streams' values at a time.
+// The merged partials of streams w0 + [b0, b1) of one (set, query head): the
+// common maximum M, the sum L and, in lane t, dims [t * D/32, (t+1) * D/32) of
+// the weighted O.  Combined in stream order: the lanes fetch 32 streams' (m, l)
+// side by side, so the maximum and every weight cost one round trip; then the
+// O of 8 streams is loaded at a time.
 template <int D>
-__global__ void __launch_bounds__(128)
-decode_merge_kernel(const Problem p, const int64_t* __restrict__ offsets, int cap, int n_streams,
-                    const float* __restrict__ part, float* __restrict__ out,
-                    uint32_t* __restrict__ status) {
+struct DecMerged {
+    float M = -INFINITY, L = 0.f, acc[D / 32] = {};
+};
+
+template <int D, typename Slot>
+__device__ __forceinline__ void dec_merge(DecMerged<D>& r, Slot slot_of, int b0, int b1, int hpp, int hh,
+                                          int lane) {
     constexpr int DPL = D / 32;
-    const int lane = threadIdx.x & 31;
-    const int n_sets = p.L * p.H_kv;
-    const int hb = blockIdx.y;
-    const int nh = min(kDecHeads, p.G - hb * kDecHeads);
-    const int hpp = decode_heads(p), rec = decode_record_floats(p);
-    const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int s = gw / hpp, hh = gw % hpp;
-    // inputs only before the wait (the first kernel writes none of them); its
-    // partial results after it, through L2
-    long long lo_raw = 0, hi_raw = 0, r0_raw = 0, r1_raw = 0;
-    if (s < n_sets) {
-        lo_raw = offsets[s];
-        hi_raw = offsets[s + 1];
-        r0_raw = offsets[0];
-        r1_raw = offsets[n_sets];
-    }
-    griddep_wait();
-    if (s >= n_sets || hh >= nh) return;
-    // every set's rows must lie in order inside [0, cap)
-    if (hh == 0 && lane == 0 && (lo_raw < 0 || hi_raw < lo_raw || hi_raw > cap))
-        raise_status(status, TGVKV_STATUS_INDEX);
-    // the first kernel's clipping and split of the rows
-    const int R0 = clampi(r0_raw, 0, cap), R1 = max(clampi(r1_raw, 0, cap), R0);
-    const int lo = min(max(clampi(lo_raw, 0, cap), R0), R1);
-    const int hi = min(max(clampi(hi_raw, 0, cap), lo), R1);
-    const int l = s / p.H_kv, gk = s % p.H_kv;
-    float* o = out + ((size_t)l * p.H_q + gk * p.G + hb * kDecHeads + hh) * D + DPL * lane;
-    if (hi <= lo) {   // an empty set gives 0
-#pragma unroll
-        for (int c = 0; c < DPL; ++c) o[c] = 0.f;
-        return;
-    }
-    const int per = (int)(((long long)R1 - R0 + n_streams - 1) / n_streams);
-    const int w0 = (lo - R0) / per, w1 = (hi - 1 - R0) / per;
-    if (w0 == w1) return;   // inside one stream: written by the first kernel
-    const bool w0_second = lo != R0 + w0 * per;
-    const int nw = w1 - w0 + 1;
-    auto slot_of = [&](int w) {
-        return dec_slot(const_cast<float*>(part), n_streams, hb, w, (w == w0 && w0_second) ? 1 : 0,
-                        rec);
-    };
-    float Lt = 0.f, acc[DPL];
-#pragma unroll
-    for (int c = 0; c < DPL; ++c) acc[c] = 0.f;
-    float M = -INFINITY;
-    for (int b = 0; b < nw; b += 32) {
-        // (m, l) of 32 streams side by side: the common maximum and the weights
-        // in one round trip (a later batch of 32 rescales what came before)
-        const int cnt = nw - b < 32 ? nw - b : 32;
+    for (int b = b0; b < b1; b += 32) {
+        // (a later batch of 32 rescales what came before)
+        const int cnt = b1 - b < 32 ? b1 - b : 32;
         float mw = -INFINITY, lw = 0.f;
         if (lane < cnt) {
-            const float* pp = slot_of(w0 + b + lane);
+            const float* pp = slot_of(b + lane);
             mw = __ldcg(pp + hpp * D + hh);
             lw = __ldcg(pp + hpp * D + hpp + hh);
         }
         float Mb = mw;
 #pragma unroll
         for (int k = 16; k > 0; k >>= 1) Mb = fmaxf(Mb, __shfl_xor_sync(~0u, Mb, k));
-        const float Mn = fmaxf(M, Mb);
+        const float Mn = fmaxf(r.M, Mb);
         if (!(Mn > -INFINITY)) continue;   // no mass yet
-        const float fa = fast_exp2(M - Mn);   // M = -inf: 0
+        const float fa = fast_exp2(r.M - Mn);   // M = -inf: 0
         // a segment without mass (m = -inf) adds nothing
         const float f = mw > -INFINITY ? fast_exp2(mw - Mn) : 0.f;
         float lf = lw * f;
 #pragma unroll
         for (int k = 16; k > 0; k >>= 1) lf += __shfl_xor_sync(~0u, lf, k);
-        Lt = Lt * fa + lf;
+        r.L = r.L * fa + lf;
 #pragma unroll
-        for (int c = 0; c < DPL; ++c) acc[c] *= fa;
-        M = Mn;
-        // the weighted O of the batch, 8 streams' loads in flight at a time
+        for (int c = 0; c < DPL; ++c) r.acc[c] *= fa;
+        r.M = Mn;
         for (int j0 = 0; j0 < cnt; j0 += 8) {
             float ov[8][DPL];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 if (j0 + u < cnt) {
-                    const float* ow = slot_of(w0 + b + j0 + u) + hh * D + DPL * lane;
+                    const float* ow = slot_of(b + j0 + u) + hh * D + DPL * lane;
                     if (DPL == 4) {
                         const float4 t = __ldcg(reinterpret_cast<const float4*>(ow));
                         ov[u][0] = t.x;
@@ -587,18 +535,106 @@ decode_merge_kernel(const Problem p, const int64_t* __restrict__ offsets, int ca
             for (int u = 0; u < 8; ++u) {
                 const float fj = __shfl_sync(~0u, f, (j0 + u) & 31);
 #pragma unroll
-                for (int c = 0; c < DPL; ++c) acc[c] += ov[u][c] * fj;
+                for (int c = 0; c < DPL; ++c) r.acc[c] += ov[u][c] * fj;
             }
         }
     }
-    const float inv = Lt > 0.f ? 1.f / Lt : 0.f;
+}
+
+// The split sets' merge, the CSR check and the empty sets: MW warps per
+// (set, query head of the pass); with MW > 1 a CTA of its own, each warp
+// merging a contiguous share of the streams, the shares then combined in order
+// from shared memory.  Launched as a programmatic dependent of decode_kernel:
+// it reads its inputs, then waits for that grid's partial results.  Results do
+// not depend on timing.
+template <int D, int MW>
+__global__ void __launch_bounds__(MW > 1 ? 32 * MW : 128)
+decode_merge_kernel(const Problem p, const int64_t* __restrict__ offsets, int cap, int n_streams,
+                    const float* __restrict__ part, float* __restrict__ out,
+                    uint32_t* __restrict__ status) {
+    constexpr int DPL = D / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_sets = p.L * p.H_kv;
+    const int hb = blockIdx.y;
+    const int nh = min(kDecHeads, p.G - hb * kDecHeads);
+    const int hpp = decode_heads(p), rec = decode_record_floats(p);
+    const int gw = MW > 1 ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + warp;
+    const int share = MW > 1 ? warp : 0;       // this warp's share of the streams
+    const int s = gw / hpp, hh = gw % hpp;
+    // inputs only before the wait (the first kernel writes none of them); its
+    // partial results after it, through L2
+    long long lo_raw = 0, hi_raw = 0, r0_raw = 0, r1_raw = 0;
+    if (s < n_sets) {
+        lo_raw = offsets[s];
+        hi_raw = offsets[s + 1];
+        r0_raw = offsets[0];
+        r1_raw = offsets[n_sets];
+    }
+    griddep_wait();
+    if (s >= n_sets || hh >= nh) return;
+    // every set's rows must lie in order inside [0, cap)
+    if (hh == 0 && share == 0 && lane == 0 && (lo_raw < 0 || hi_raw < lo_raw || hi_raw > cap))
+        raise_status(status, TGVKV_STATUS_INDEX);
+    // the first kernel's clipping and split of the rows
+    const int R0 = clampi(r0_raw, 0, cap), R1 = max(clampi(r1_raw, 0, cap), R0);
+    const int lo = min(max(clampi(lo_raw, 0, cap), R0), R1);
+    const int hi = min(max(clampi(hi_raw, 0, cap), lo), R1);
+    const int l = s / p.H_kv, gk = s % p.H_kv;
+    float* o = out + ((size_t)l * p.H_q + gk * p.G + hb * kDecHeads + hh) * D + DPL * lane;
+    if (hi <= lo) {   // an empty set gives 0
+        if (share == 0)
 #pragma unroll
-    for (int c = 0; c < DPL; ++c) o[c] = acc[c] * inv;
+            for (int c = 0; c < DPL; ++c) o[c] = 0.f;
+        return;
+    }
+    const int per = (int)(((long long)R1 - R0 + n_streams - 1) / n_streams);
+    const int w0 = (lo - R0) / per, w1 = (hi - 1 - R0) / per;
+    if (w0 == w1) return;   // inside one stream: written by the first kernel
+    const bool w0_second = lo != R0 + w0 * per;
+    const int nw = w1 - w0 + 1;
+    auto slot_of = [&](int b) {      // stream w0 + b
+        return dec_slot(const_cast<float*>(part), n_streams, hb, w0 + b, (b == 0 && w0_second) ? 1 : 0,
+                        rec);
+    };
+    DecMerged<D> r;
+    if (MW == 1) {
+        dec_merge<D>(r, slot_of, 0, nw, hpp, hh, lane);
+    } else {
+        __shared__ float sm[MW], sl[MW];
+        __shared__ float so[MW][D];
+        const int each = (nw + MW - 1) / MW;
+        const int b0 = min(share * each, nw);
+        dec_merge<D>(r, slot_of, b0, min(b0 + each, nw), hpp, hh, lane);
+        if (lane == 0) {
+            sm[share] = r.M;
+            sl[share] = r.L;
+        }
+#pragma unroll
+        for (int c = 0; c < DPL; ++c) so[share][DPL * lane + c] = r.acc[c];
+        __syncthreads();
+        if (share != 0) return;
+        r = DecMerged<D>();
+#pragma unroll
+        for (int w = 0; w < MW; ++w) r.M = fmaxf(r.M, sm[w]);
+#pragma unroll
+        for (int w = 0; w < MW; ++w) {
+            const float f = sm[w] > -INFINITY ? fast_exp2(sm[w] - r.M) : 0.f;
+            r.L += sl[w] * f;
+#pragma unroll
+            for (int c = 0; c < DPL; ++c) r.acc[c] += so[w][DPL * lane + c] * f;
+        }
+    }
+    const float inv = r.L > 0.f ? 1.f / r.L : 0.f;
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) o[c] = r.acc[c] * inv;
 }
 
 // Rows per chunk and streams (warps) per CTA.
 constexpr int kDecCH = 16;
 constexpr int kDecW = 8;
+// Warps that merge one (set, query head) when the sets are few, and the mean
+// number of streams per set from which they do.
+constexpr int kDecMergeWarps = 16, kDecMergeSplit = 16;
 
 template <int D, int CH, int W>
 cudaError_t launch_dec(const Problem& p, const uint16_t* q, const uint16_t* k_rows,
@@ -632,8 +668,13 @@ cudaError_t launch_dec(const Problem& p, const uint16_t* q, const uint16_t* k_ro
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the merge, as a programmatic dependent: it is scheduled while the first
     // kernel runs and waits on the device for its results
-    const long long warps = (long long)n_sets * decode_heads(p);
-    return launch_dependent(decode_merge_kernel<D>, dim3((unsigned)((warps + 3) / 4), decode_passes(p)),
+    const long long merges = (long long)n_sets * decode_heads(p);
+    if (ctas * W >= kDecMergeSplit * n_sets)
+        return launch_dependent(decode_merge_kernel<D, kDecMergeWarps>,
+                                dim3((unsigned)merges, decode_passes(p)), dim3(32 * kDecMergeWarps), 0,
+                                stream, p, offsets, cap, ctas * W, static_cast<const float*>(part), out,
+                                status);
+    return launch_dependent(decode_merge_kernel<D, 1>, dim3((unsigned)((merges + 3) / 4), decode_passes(p)),
                             dim3(128), 0, stream, p, offsets, cap, ctas * W,
                             static_cast<const float*>(part), out, status);
 }
