@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes
 import math
 from dataclasses import dataclass
+from functools import lru_cache
 
 import torch
 
@@ -64,13 +65,17 @@ def desc_for_workload(wl, softmax_scale=0.0, **options) -> Desc:
 
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the raw handle of torch.cuda.current_stream(), without building the object
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
-        return ctypes.c_void_p(stream.cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _ptr(t, dtypes, numel, name):
+    """The device address of a tensor that holds what the call needs (None: NULL)."""
     if t is None:
         return None
     if not isinstance(t, torch.Tensor):
@@ -83,7 +88,7 @@ def _ptr(t, dtypes, numel, name):
         raise ValueError(f"{name} must be contiguous")
     if t.numel() < numel:
         raise ValueError(f"{name} holds {t.numel()} elements, needs {numel}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _check(code, fn):
@@ -91,11 +96,26 @@ def _check(code, fn):
         raise TgvkvError(code, fn)
 
 
-def tgvkv_workspace_size(desc: Desc) -> int:
-    n = _lib.load().tgvkv_workspace_size(ctypes.byref(desc))
+# Every call checks its buffers against these two sizes; they follow from the
+# descriptor's values alone, so the recent ones are remembered by value.
+@lru_cache(maxsize=256)
+def _workspace_size(desc: bytes) -> int:
+    n = _lib.load().tgvkv_workspace_size(ctypes.byref(Desc.from_buffer_copy(desc)))
     if n == 0:
         raise TgvkvError(-1, "tgvkv_workspace_size")
     return int(n)
+
+
+@lru_cache(maxsize=256)
+def _retained_rows(desc: bytes, ratio: float) -> int:
+    n = _lib.load().tgvkv_retained_rows(ctypes.byref(Desc.from_buffer_copy(desc)), ratio)
+    if n < 0:
+        raise TgvkvError(-1, "tgvkv_retained_rows")
+    return int(n)
+
+
+def tgvkv_workspace_size(desc: Desc) -> int:
+    return _workspace_size(bytes(desc))
 
 
 def tgvkv_vision_budget_total(desc: Desc, ratio: float) -> int:
@@ -113,10 +133,7 @@ def tgvkv_budget_total(desc: Desc, ratio: float) -> int:
 
 
 def tgvkv_retained_rows(desc: Desc, ratio: float) -> int:
-    n = _lib.load().tgvkv_retained_rows(ctypes.byref(desc), float(ratio))
-    if n < 0:
-        raise TgvkvError(-1, "tgvkv_retained_rows")
-    return int(n)
+    return _retained_rows(bytes(desc), float(ratio))
 
 
 def tgvkv_workspace_init(desc: Desc, ws: torch.Tensor, stream=None):

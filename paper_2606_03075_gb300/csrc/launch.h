@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace tgvkv {
@@ -28,6 +30,22 @@ cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
+}
+
+// Whether the kernel was compiled to `regs` registers per thread: one that splits
+// its registers between warpgroups (setmaxnreg) may only be launched with the
+// count its split adds up to.  (A property of the built code: asked until known.)
+template <auto Kern>
+bool has_registers(int regs) {
+    static std::atomic<int> known{-1};
+    int n = known.load(std::memory_order_relaxed);
+    if (n < 0) {
+        cudaFuncAttributes attr;
+        if (cudaFuncGetAttributes(&attr, Kern) != cudaSuccess) return false;
+        n = attr.numRegs;
+        known.store(n, std::memory_order_relaxed);
+    }
+    return n == regs;
 }
 
 // TWR scores + TVB statistic (score_tc.cu).  The completion counters in the

@@ -145,15 +145,6 @@ __device__ __forceinline__ bool warp_wait_all(uint64_t* bar, uint32_t parity, vo
     return __all_sync(~0u, got);
 }
 
-template <int REGS>
-__device__ __forceinline__ void regs_inc() {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
-}
-template <int REGS>
-__device__ __forceinline__ void regs_dec() {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&b);
@@ -366,7 +357,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
 
     if (warp < OUT_WARP) {
         // -------------------------------------------------------- softmax
-        regs_inc<SOFT_REGS>();
+        tc::regs_inc<SOFT_REGS>();
         tc::named_bar_sync(2, LOAD_WARP * 32);   // the output warps' tables
         const int w = warp >> 2, quarter = warp & 3;         // stream, lane quarter
         const int r = quarter * 32 + lane;                   // this thread's row = TMEM lane
@@ -491,7 +482,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         if (!ok) raise_status(status, TGVKV_STATUS_TIMEOUT);
     } else if (warp < LOAD_WARP) {
         // -------------------------------------------------------- output rows
-        regs_dec<OUT_REGS>();
+        tc::regs_dec<OUT_REGS>();
         // The tables: the query rows of each row tile t, indices wtile[t] ..
         // wtile[t + 1] of text_pos (positions ascend), as the first row at or after
         // position 128 t; their positions as bits; and the modality as bits, whole
@@ -589,7 +580,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         }
         if (!ok) raise_status(status, TGVKV_STATUS_TIMEOUT);
     } else {
-        regs_dec<ROLE_REGS>();
+        tc::regs_dec<ROLE_REGS>();
         if (warp == LOAD_WARP && lane == 0) {
             // ---------------------------------------------------- producer
             tc::tma_prefetch_desc(&tmap_q);
@@ -951,10 +942,7 @@ cudaError_t launch_prefill_d(const Problem& p, const uint16_t* q, const uint16_t
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // the register split adds up only for the register count it was written for
-    cudaFuncAttributes attr;
-    e = cudaFuncGetAttributes(&attr, prefill_kernel<D, SOLO>);
-    if (e != cudaSuccess) return e;
-    if (attr.numRegs != P_REGS) return cudaErrorInvalidConfiguration;
+    if (!has_registers<prefill_kernel<D, SOLO>>(P_REGS)) return cudaErrorInvalidConfiguration;
     const int n_qt = (p.N + PM - 1) / PM;
     const int n_items = p.L * p.H_q * (SOLO ? n_qt : (n_qt + 1) / 2);
     // heads worked on together: whole KV groups whose K and V fit kBatchBytes
