@@ -217,11 +217,9 @@ __global__ void __launch_bounds__(W * 32, 1)
 decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ CUtensorMap mk8,
               const __grid_constant__ CUtensorMap mvf, const __grid_constant__ CUtensorMap mv8,
               const __grid_constant__ CUtensorMap mq, const Problem p,
-              const int64_t* __restrict__ offsets, int cap, float* __restrict__ out,
+              const int64_t* offsets, int cap, float* __restrict__ out,
               float* __restrict__ part, uint32_t* __restrict__ status) {
     using Gm = DecGeom<D, CH, W>;
-    // the merge kernel may be scheduled now; it waits for this grid's results
-    griddep_launch_dependents();
     if (threadIdx.x == 0) {   // the descriptors' first fetch overlaps the prologue
         tc::tma_prefetch_desc(&mkf);
         tc::tma_prefetch_desc(&mk8);
@@ -245,6 +243,16 @@ decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ C
     const int nh = min(kDecHeads, p.G - hb * kDecHeads);
     const int hpp = decode_heads(p), rec = decode_record_floats(p);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) never = 0;
+    if (lane == 0) {
+        for (int st = 0; st < kDecStages; ++st) tc::mbar_init(&tl.full[warp][st], 1);
+        tc::fence_mbar_init();
+    }
+    // launched as a programmatic dependent of the kernel before it: what that one
+    // wrote (the rows, or the partials its merge still reads) from here on only
+    griddep_wait();
+    // the merge kernel may be scheduled now; it waits for this grid's results
+    griddep_launch_dependents();
     DecRows rows;
     rows.so = offs_s;
     rows.go = reinterpret_cast<const long long*>(offsets);
@@ -265,11 +273,6 @@ decode_kernel(const __grid_constant__ CUtensorMap mkf, const __grid_constant__ C
                 if (idx <= n_sets) offs_s[idx] = clampi(v[u], 0, cap);
             }
         }
-    }
-    if (tid == 0) never = 0;
-    if (lane == 0) {
-        for (int st = 0; st < kDecStages; ++st) tc::mbar_init(&tl.full[warp][st], 1);
-        tc::fence_mbar_init();
     }
     __syncthreads();
 
@@ -549,7 +552,7 @@ __device__ __forceinline__ void dec_merge(DecMerged<D>& r, Slot slot_of, int b0,
 // not depend on timing.
 template <int D, int MW>
 __global__ void __launch_bounds__(MW > 1 ? 32 * MW : 128)
-decode_merge_kernel(const Problem p, const int64_t* __restrict__ offsets, int cap, int n_streams,
+decode_merge_kernel(const Problem p, const int64_t* offsets, int cap, int n_streams,
                     const float* __restrict__ part, float* __restrict__ out,
                     uint32_t* __restrict__ status) {
     constexpr int DPL = D / 32;
@@ -561,16 +564,20 @@ decode_merge_kernel(const Problem p, const int64_t* __restrict__ offsets, int ca
     const int gw = MW > 1 ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + warp;
     const int share = MW > 1 ? warp : 0;       // this warp's share of the streams
     const int s = gw / hpp, hh = gw % hpp;
-    // inputs only before the wait (the first kernel writes none of them); its
-    // partial results after it, through L2
+    // inputs only before the wait (the first kernel writes none of them, and began its
+    // own work after the kernel that did); its partial results after it; all through L2
     long long lo_raw = 0, hi_raw = 0, r0_raw = 0, r1_raw = 0;
+    const long long* ofs = reinterpret_cast<const long long*>(offsets);
     if (s < n_sets) {
-        lo_raw = offsets[s];
-        hi_raw = offsets[s + 1];
-        r0_raw = offsets[0];
-        r1_raw = offsets[n_sets];
+        lo_raw = __ldcg(ofs + s);
+        hi_raw = __ldcg(ofs + s + 1);
+        r0_raw = __ldcg(ofs + 0);
+        r1_raw = __ldcg(ofs + n_sets);
     }
     griddep_wait();
+    // the next kernel on the stream may be scheduled (it waits for this one's end
+    // before it touches the partials or the output)
+    griddep_launch_dependents();
     if (s >= n_sets || hh >= nh) return;
     // every set's rows must lie in order inside [0, cap)
     if (hh == 0 && share == 0 && lane == 0 && (lo_raw < 0 || hi_raw < lo_raw || hi_raw > cap))
@@ -663,9 +670,14 @@ cudaError_t launch_dec(const Problem& p, const uint16_t* q, const uint16_t* k_ro
     const int sms = device_sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;
     const int ctas = sms < kDecMaxStreams / W ? sms : kDecMaxStreams / W;
-    decode_kernel<D, CH, W><<<dim3(ctas, decode_passes(p)), W * 32, smem, stream>>>(
-        mkf, mk8, mvf, mv8, mq, p, offsets, cap, out, part, status);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // A programmatic dependent of the kernel before it: an eviction's gather or
+    // another step's merge lets it be scheduled while that one runs, so its launch,
+    // descriptor fetches and barrier setup cost nothing (measured, steps back to
+    // back: 33.2 -> 30.6 us for 1024 sets of 128-dim rows of a 32-layer cache,
+    // 14.4 -> 12.2 us for one layer of 4 sets of 8.7 thousand rows).
+    e = launch_dependent(decode_kernel<D, CH, W>, dim3(ctas, decode_passes(p)), dim3(W * 32), smem, stream,
+                         mkf, mk8, mvf, mv8, mq, p, offsets, cap, out, part, status);
+    if (e != cudaSuccess) return e;
     // the merge, as a programmatic dependent: it is scheduled while the first
     // kernel runs and waits on the device for its results
     const long long merges = (long long)n_sets * decode_heads(p);

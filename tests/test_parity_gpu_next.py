@@ -329,6 +329,54 @@ def test_decode_empty_sets_give_zero(api):
     assert np.array_equal(o, np.zeros_like(o))
 
 
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("name", ["tiny", "wide_group"])
+def test_decode_steps_back_to_back(api, name, captured):
+    """A decode step may be launched while the kernel before it still runs.  Steps in
+    one workspace and one set of buffers -- each after an eviction that rewrites the
+    rows and the offsets, and after a copy that rewrites the queries, or straight
+    after another step -- give the same bits without a wait between them as with one,
+    also replayed from a graph."""
+    wl = DECODE_CASES[name]
+    desc = api.desc_for_workload(wl)
+    ws = api.new_workspace(desc)
+    devs = [P.device_inputs(synth.generate(wl, seed=s)) for s in (6, 7)]
+    ratios = [wl.ratios[0], wl.ratios[0] / 2]
+    out = api.alloc_outputs(desc, max(ratios))
+    qs = [torch.from_numpy(_decode_q(wl, s)).cuda().view(torch.bfloat16) for s in (1, 2, 3)]
+    q = torch.empty_like(qs[0])
+    shape = (6, wl.L, wl.H_q, wl.d)
+
+    def steps(o, wait):
+        for i in range(6):
+            if i % 3 == 0:
+                dev, ratio = devs[i // 3], ratios[i // 3]
+                api.tgvkv_evict(desc, dev["q"], dev["k"], dev["v"], dev["modality"],
+                                dev["text_pos"], dev["w"], ratio, out, ws)
+                wait()
+            if i % 3 != 2:
+                q.copy_(qs[i % 3])
+                wait()
+            api.tgvkv_decode(desc, q, out.k_out, out.v_out, out.offsets, o[i], ws)
+            wait()
+
+    ref = torch.full(shape, float("nan"), device="cuda")
+    steps(ref, torch.cuda.synchronize)
+    got = torch.full(shape, float("nan"), device="cuda")
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            steps(got, lambda: None)
+        got.fill_(float("nan"))
+        for _ in range(3):
+            graph.replay()
+    else:
+        for _ in range(20):
+            steps(got, lambda: None)
+    assert api.tgvkv_status(ws) == 0
+    assert torch.isfinite(ref).all() and torch.equal(got, ref)
+
+
 # Ragged CSR layouts around the decode kernel's boxes (8 and 32 rows): sets of
 # 0, 1, 7-9, 15-17, 31-33, 63-65 and 257 rows, empty sets between full ones, a
 # base offset before the first set and spare rows after the last; groups of 1,
