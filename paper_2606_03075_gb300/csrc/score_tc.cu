@@ -491,8 +491,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     }
 
     // ------------------------------------------------------------ MMA issuers
-    // Step k goes to issuer k & 1 and accumulator k & 1.
-    if ((warp == 1 || warp == MMA2_WARP) && lane == 0) {
+    // Step k goes to issuer k & 1 and accumulator k & 1.  The whole warp walks the
+    // steps and one elected lane issues: the operands then stay in uniform registers.
+    // (From a branch on the lane they are moved there before every MMA, 110 cycles
+    // apart instead of the 64 that a 128 x 128 x 16 product takes; 28 layers x 4 KV
+    // heads x 4352 keys, Eq. 7 weights: 551 -> 542 us; 28 layers, 1920 query rows x
+    // 8.2 thousand keys: 1535 -> 1493 us.)
+    if (warp == 1 || warp == MMA2_WARP) {
         const int me = warp == 1 ? 0 : 1;
         // shared-memory descriptors, computed once: the start-address field
         // (16-byte units, < 2^14 inside 256 KB) takes plain additions
@@ -504,12 +509,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         bool ok = true;
         for (int n = 0; ok; ++n) {
             const int slot = n % NIQ;
-            if (!tc::mbar_wait(&s.it_full[slot], (n / NIQ) & 1, abort_flag)) {
+            if (!warp_wait(&s.it_full[slot], (n / NIQ) & 1, abort_flag)) {
                 ok = false;
                 break;
             }
             const int id = s.item_q[slot];
-            tc::mbar_arrive(&s.it_empty[slot]);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&s.it_empty[slot]);
             if (id < 0) break;
             const Item itm = item_info(p, s, mode, id, n_two);
             const int nslot = mode == MODE_PAIR ? itm.nparts : 1;
@@ -517,7 +523,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             for (int r = 0; r < nslot; ++r) {
                 const int qs = mode == MODE_PAIR ? r : qs0;
                 const int use = qs ? qn1++ : qn0++;
-                if (!tc::mbar_wait(&s.q_full[qs], use & 1, abort_flag)) {
+                if (!warp_wait(&s.q_full[qs], use & 1, abort_flag)) {
                     ok = false;
                     break;
                 }
@@ -533,59 +539,64 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     const bool has2 = kt[1] >= 0;
                     if ((step & 1) == me) {
                         const int b = step & 1;
-                        bool got = tc::mbar_wait(&s.full[it % STAGES], (it / STAGES) & 1, abort_flag);
+                        bool got = warp_wait(&s.full[it % STAGES], (it / STAGES) & 1, abort_flag);
                         if (got && nst == 2)
-                            got = tc::mbar_wait(&s.full[(it + 1) % STAGES], ((it + 1) / STAGES) & 1,
+                            got = warp_wait(&s.full[(it + 1) % STAGES], ((it + 1) / STAGES) & 1,
                                                 abort_flag);
-                        if (got) got = tc::mbar_wait(&s.s_empty[b], ((step >> 1) & 1) ^ 1, abort_flag);
+                        if (got) got = warp_wait(&s.s_empty[b], ((step >> 1) & 1) ^ 1, abort_flag);
                         if (!got) {
                             ok = false;
                             break;
                         }
                         tc::fence_after_sync();
-                        const uint32_t d = tmem + (uint32_t)(b * SCOLS);
-                        const uint64_t k0 = kdesc0 + (uint64_t)((it % STAGES) * KSTAGE_DESC);
-                        const uint64_t k1 = kdesc0 + (uint64_t)(((it + 1) % STAGES) * KSTAGE_DESC);
-                        if (mode == MODE_PAIR) {
-                            if (pass == 0) {
-                                if (kt[0] < itm.nt[0])
-                                    mma_block<D>(d, qd, Q_HALF, k0, K_HALF, IDESC128);
-                                if (itm.nparts == 2 && kt[0] < itm.nt[1])
-                                    mma_block<D>(d + BN, qd + Q_SLOT, Q_HALF, k0, K_HALF, IDESC128);
-                            } else if (itm.nparts == 2) {
-                                mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC256);
+                        if (tc::elect_one()) {
+                            const uint32_t d = tmem + (uint32_t)(b * SCOLS);
+                            const uint64_t k0 = kdesc0 + (uint64_t)((it % STAGES) * KSTAGE_DESC);
+                            const uint64_t k1 = kdesc0 + (uint64_t)(((it + 1) % STAGES) * KSTAGE_DESC);
+                            if (mode == MODE_PAIR) {
+                                if (pass == 0) {
+                                    if (kt[0] < itm.nt[0])
+                                        mma_block<D>(d, qd, Q_HALF, k0, K_HALF, IDESC128);
+                                    if (itm.nparts == 2 && kt[0] < itm.nt[1])
+                                        mma_block<D>(d + BN, qd + Q_SLOT, Q_HALF, k0, K_HALF, IDESC128);
+                                } else if (itm.nparts == 2) {
+                                    mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC256);
+                                } else {
+                                    mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC128);
+                                }
+                            } else if (pass == 0) {
+                                // Q against both adjacent K stages in one N = 256 product
+                                mma_block<D>(d, qd, Q_HALF, k0, K_HALF, has2 ? IDESC256 : IDESC128);
+                            } else if (mode == MODE_PACKED) {
+                                // head h's rows are Q rows 64h..64h+63 (64 rows = 8 KB = 512 units on)
+                                mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC64);
+                                if (has2) mma_block<D>(d + BN + 64, k1, K_HALF, qd + 512, Q_HALF, IDESC64);
                             } else {
                                 mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC128);
+                                if (has2) mma_block<D>(d + BN, k1, K_HALF, qd, Q_HALF, IDESC128);
                             }
-                        } else if (pass == 0) {
-                            // Q against both adjacent K stages in one N = 256 product
-                            mma_block<D>(d, qd, Q_HALF, k0, K_HALF, has2 ? IDESC256 : IDESC128);
-                        } else if (mode == MODE_PACKED) {
-                            // head h's rows are Q rows 64h..64h+63 (64 rows = 8 KB = 512 units on)
-                            mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC64);
-                            if (has2) mma_block<D>(d + BN + 64, k1, K_HALF, qd + 512, Q_HALF, IDESC64);
-                        } else {
-                            mma_block<D>(d, k0, K_HALF, qd, Q_HALF, IDESC128);
-                            if (has2) mma_block<D>(d + BN, k1, K_HALF, qd, Q_HALF, IDESC128);
+                            tc::mma_commit(&s.s_full[b]);
+                            tc::mma_commit(&s.empty[it % STAGES]);
+                            if (nst == 2) tc::mma_commit(&s.empty[(it + 1) % STAGES]);
                         }
-                        tc::mma_commit(&s.s_full[b]);
-                        tc::mma_commit(&s.empty[it % STAGES]);
-                        if (nst == 2) tc::mma_commit(&s.empty[(it + 1) % STAGES]);
+                        __syncwarp();
                     }
                     it += nst;
                     ++step;
                 }
             }
             // the item's Q slots are free once both issuers' MMAs have finished
-            for (int r = 0; r < nslot; ++r) tc::mma_commit(&s.q_empty[mode == MODE_PAIR ? r : qs0]);
+            if (tc::elect_one())
+                for (int r = 0; r < nslot; ++r) tc::mma_commit(&s.q_empty[mode == MODE_PAIR ? r : qs0]);
         }
         if (!ok) {
             s.abort_flag = 1;
-            raise_status(status, TGVKV_STATUS_TIMEOUT);
+            if (lane == 0) raise_status(status, TGVKV_STATUS_TIMEOUT);
         }
         // every MMA this CTA issued has finished before TMEM is released
-        tc::mma_commit(&s.mma_done);
-        tc::mbar_wait(&s.mma_done, 0, &s.never);
+        if (tc::elect_one()) tc::mma_commit(&s.mma_done);
+        __syncwarp();
+        warp_wait(&s.mma_done, 0, &s.never);
     }
 
     // ------------------------------------------------------------ softmax
