@@ -117,6 +117,28 @@ __device__ __forceinline__ void exp_word_both(const float (&x)[32], float sl2, f
     }
 }
 
+// a + c += the sum of 2^(x_c sl2 + nm) over 16 columns, sums left apart.
+__device__ __forceinline__ void exp_sum16(const float (&x)[16], float sl2, float nm, float2& a,
+                                          float2& c) {
+    const float2 s2 = make_float2(sl2, sl2), n2 = make_float2(nm, nm);
+#pragma unroll
+    for (int e = 0; e < 16; e += 4) {
+        const float2 t0 = fma2(make_float2(x[e], x[e + 1]), s2, n2);
+        const float2 t1 = fma2(make_float2(x[e + 2], x[e + 3]), s2, n2);
+        a = add2(a, make_float2(fast_exp2(t0.x), fast_exp2(t0.y)));
+        c = add2(c, make_float2(fast_exp2(t1.x), fast_exp2(t1.y)));
+    }
+}
+
+__device__ __forceinline__ float max16(const float (&x)[16]) {
+    float a = fmax3(x[0], x[1], x[2]), b = fmax3(x[3], x[4], x[5]);
+    a = fmax3(a, x[6], x[7]);
+    b = fmax3(b, x[8], x[9]);
+    a = fmax3(a, x[10], x[11]);
+    b = fmax3(b, x[12], x[13]);
+    return fmax3(fmaxf(a, b), x[14], x[15]);
+}
+
 // Online statistics of one row over one 32-key word: columns 0..lim visible.
 // The row keeps a reference m (base-2 units) and sums its terms 2^(x sl2 - m):
 // the row's first visible word sets m to that word's maximum; a later word
@@ -124,7 +146,8 @@ __device__ __forceinline__ void exp_word_both(const float (&x)[32], float sl2, f
 // or overflowed), and is then taken again against its own maximum, which moves
 // m up (z and v rescaled).  Any reference gives the same attention entries
 // 2^(x sl2 - m) / Z; this one never exceeds the row's maximum and keeps every
-// term at most kWordSumLimit, and most words skip the 32-key maximum.
+// term at most kWordSumLimit, and most words skip the 32-key maximum.  (The pair
+// items of the score kernel hold the limit against 48 and 16 keys at a time.)
 constexpr float kWordSumLimit = 32.f * 256.f;
 
 __device__ __forceinline__ void row_word(const float (&x)[32], float sl2, int lim, uint32_t vm,

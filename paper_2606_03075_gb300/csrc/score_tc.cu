@@ -102,6 +102,7 @@ struct PSmem {
     int row_q[2][BM];                        // ... its global Q row, -1 = none
     alignas(16) float row_nmp[2][BM];        // -(m_i - log2 c_i); -inf = no row
     float row_w[2][BM], row_mass[2][BM];
+    int grp_min[2][4], grp_max[2][4];        // least / largest position of a slot's 32-lane group
     float part_m[4][BM], part_z[4][BM], part_v[4][BM], part_u[4][BM];
     int item_q[NIQ];
     uint32_t tmem_base;
@@ -237,6 +238,21 @@ __device__ __forceinline__ float colsum_group(const float (&y)[32], const float*
         }
     }
     return (a.x + a.y) + (b.x + b.y);
+}
+
+// a + c += the sum over 16 rows of 2^(y_i sl2 + nmp_i): colsum_group of rows that
+// all exist and see the key, sums left apart.
+__device__ __forceinline__ void colsum16(const float (&y)[16], const float* nmp, float sl2, float2& a,
+                                         float2& c) {
+    const float2 s2 = make_float2(sl2, sl2);
+#pragma unroll
+    for (int e = 0; e < 16; e += 4) {
+        const float4 n4 = *reinterpret_cast<const float4*>(nmp + e);
+        const float2 t0 = fma2(make_float2(y[e], y[e + 1]), s2, make_float2(n4.x, n4.y));
+        const float2 t1 = fma2(make_float2(y[e + 2], y[e + 3]), s2, make_float2(n4.z, n4.w));
+        a = add2(a, make_float2(fast_exp2(t0.x), fast_exp2(t0.y)));
+        c = add2(c, make_float2(fast_exp2(t1.x), fast_exp2(t1.y)));
+    }
 }
 
 // A bounded wait whose outcome is the same for every lane of the warp (the
@@ -631,6 +647,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const int id = s.cur_item;
             if (id < 0) break;
             const Item itm = item_info(p, s, mode, id, n_two);
+            // pair: key tiles, and rows per lane group, of this warp's row tile
+            const int ntA = (wi >> 1) < itm.nparts ? Item::pick(itm.nt, wi >> 1) : 0;
+            const int rpgB = Item::pick(itm.rpg, wi >> 1);
 
             // ---- rows: lane 32q + i of row slot rs holds the part's row q*rpg + i
             // (packed: lanes 64h + 32q' + i hold head h's row q'*rpg + i)
@@ -666,6 +685,14 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 s.row_pos[rs][ln] = pos;
                 s.row_w[rs][ln] = wr;
                 s.row_q[rs][ln] = has ? Item::pick(itm.qy, part) + row : -1;
+                if (mode == MODE_PAIR) {
+                    const int gmin = __reduce_min_sync(~0u, pos < 0 ? INT_MAX : pos);
+                    const int gmax = __reduce_max_sync(~0u, pos);
+                    if (lane == 0) {
+                        s.grp_min[rs][quarter] = gmin;
+                        s.grp_max[rs][quarter] = gmax;
+                    }
+                }
             }
             // the item's output rows start at zero: pass B adds two partial sums per key
             for (int r = 0; r < itm.nparts; ++r) {
@@ -688,7 +715,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 // (then doing nothing), so that the warps of a quarter always meet
                 // at the same named barriers.
                 int cur = 0, kt[2];
-                while (next_step(itm, mode, 0, cur, s.vis_before, kt, p.stats_given)) {
+                const int nA = p.stats_given ? 0 : itm.ntmax;
+                while (mode == MODE_PAIR ? cur < nA
+                                         : next_step(itm, mode, 0, cur, s.vis_before, kt, p.stats_given)) {
+                    uint32_t vm0 = 0, vm1 = 0;
+                    if (mode == MODE_PAIR) {
+                        kt[0] = cur++;
+                        vm0 = s.vmask[kt[0]][2 * (wi & 1)];
+                        vm1 = s.vmask[kt[0]][2 * (wi & 1) + 1];
+                    }
                     const int b = step & 1;
                     ++step;
                     if (ok && !warp_wait(&s.s_full[b], ((step - 1) >> 1) & 1, abort_flag)) {
@@ -702,7 +737,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                     if (mode == MODE_PAIR) {
                         blk = wi >> 1;
                         ktile = kt[0];
-                        act = blk < itm.nparts && ktile < Item::pick(itm.nt, blk);
+                        act = ktile < ntA;
                         cbase = 64 * (wi & 1);
                         nch = 2;
                     } else if (mode == MODE_SINGLE) {
@@ -722,7 +757,63 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         release_acc(&s.s_empty[b], lane);
                     } else {
                         const uint32_t ta = tq + (uint32_t)(b * SCOLS + blk * BN + cbase);
-                        for (int ch = 0; ch < nch; ++ch) {
+                        // 64 keys that every row of the warp sees, vision or not word by
+                        // word, with a reference m in every row: no branch, and each 16
+                        // columns' load in flight while the 16 before are summed.  The
+                        // accumulator is kept until the first 48 terms prove the
+                        // references good enough; else the words are taken one by one.
+                        // With the same in pass B (28 layers x 4 KV heads x 4352 keys, Eq. 7
+                        // weights): 542 -> 500 us; pass B alone 526.  Items of one row tile
+                        // stay with whole words: 5 steps an item, and 383 -> 410 us for 32
+                        // layers x 32 heads x 96 rows x 3008 keys that way.
+                        bool done = false;
+                        const bool plain =
+                            my_pos < 0 || (my_pos - (ktile * BN + cbase) >= 63 && m != -INFINITY);
+                        if (mode == MODE_PAIR && (vm0 + 1u) <= 1u && (vm1 + 1u) <= 1u &&
+                            __all_sync(~0u, plain)) {
+                            const float nm = my_pos < 0 ? -INFINITY : -m;   // no row: every term 0
+                            float2 a = make_float2(0.f, 0.f), c = a, d = a, f = a;
+                            float x0[16], x1[16];
+                            tc::tmem_ld16(ta, x0);
+                            tc::tmem_wait_ld16(x0);
+                            tc::tmem_ld16(ta + 16, x1);
+                            exp_sum16(x0, sl2, nm, a, c);
+                            tc::tmem_wait_ld16(x1);
+                            tc::tmem_ld16(ta + 32, x0);
+                            exp_sum16(x1, sl2, nm, a, c);
+                            tc::tmem_wait_ld16(x0);
+                            tc::tmem_ld16(ta + 48, x1);
+                            exp_sum16(x0, sl2, nm, d, f);
+                            const float z0 = (a.x + a.y) + (c.x + c.y);
+                            float z1 = (d.x + d.y) + (f.x + f.y);
+                            tc::tmem_wait_ld16(x1);
+                            done = __all_sync(~0u, my_pos < 0 || z0 + z1 <= kWordSumLimit);
+                            if (done) {
+                                release_acc(&s.s_empty[b], lane);
+                                z += z0;
+                                if (vm0) v += z0; else u += z0;
+                                d = f = make_float2(0.f, 0.f);
+                                exp_sum16(x1, sl2, nm, d, f);
+                                float z2 = (d.x + d.y) + (f.x + f.y);
+                                if (my_pos >= 0 && !(z2 <= kWordSumLimit)) {
+                                    // again against their own maximum
+                                    const float m_new = fmaxf(m, max16(x1) * sl2);
+                                    const float alpha = fast_exp2(m - m_new);
+                                    z *= alpha;
+                                    v *= alpha;
+                                    u *= alpha;
+                                    z1 *= alpha;
+                                    d = f = make_float2(0.f, 0.f);
+                                    exp_sum16(x1, sl2, -m_new, d, f);
+                                    z2 = (d.x + d.y) + (f.x + f.y);
+                                    m = m_new;
+                                }
+                                z1 += z2;
+                                z += z1;
+                                if (vm1) v += z1; else u += z1;
+                            }
+                        }
+                        for (int ch = done ? nch : 0; ch < nch; ++ch) {
                             float x[32];
                             tc::tmem_ld32(ta + (uint32_t)(ch * 32), x);
                             tc::tmem_wait_ld();
@@ -813,8 +904,25 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             // Pair items write one partial row per row tile.
             {
                 int cur = 0, kt[2];
+                // pair: this warp's partial row, and the least position of its 64 rows
+                // (-1 when some of them do not exist)
+                float* const out_row =
+                    score_part + ((size_t)itm.lh[0] * p.T + 2 * itm.pidx + (wi >> 1)) * p.N_v;
+                const int gmin = mode == MODE_PAIR && rpgB >= 32
+                                     ? min(s.grp_min[wi >> 1][2 * (wi & 1)],
+                                           s.grp_min[wi >> 1][2 * (wi & 1) + 1])
+                                     : -1;
                 while (next_step(itm, mode, 1, cur, s.vis_before, kt, p.stats_given)) {
                     const int b = step & 1;
+                    uint32_t word0 = 0;
+                    int vr0 = 0;
+                    bool all64 = false;
+                    if (mode == MODE_PAIR) {
+                        word0 = s.vmask[kt[0]][quarter];
+                        all64 = kt[0] * BN + BN - 1 <= gmin;
+                        vr0 = s.vq[kt[0]][quarter] + __popc(word0 & lt_mask);
+                        if (!((word0 >> lane) & 1u) || kt[0] >= ntA) vr0 = INT_MAX;
+                    }
                     if (ok && !warp_wait(&s.s_full[b], (step >> 1) & 1, abort_flag)) {
                         ok = false;
                         s.abort_flag = 1;
@@ -826,11 +934,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         blk = 0;
                         ktile = kt[0];
                         rs = wi >> 1;
-                        act = rs < itm.nparts && ktile < Item::pick(itm.nt, rs);
+                        act = ktile < ntA;
                         ccol = 64 * wi;
                         rcol = 64 * (wi & 1);
                         nch = 2;
-                        rpg = Item::pick(itm.rpg, rs);
+                        rpg = rpgB;
                         minp = Item::pick(itm.minp, rs);
                     } else if (mode == MODE_SINGLE) {
                         blk = wi >> 1;
@@ -860,29 +968,65 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         release_acc(&s.s_empty[b], lane);
                     } else {
                         const int j = ktile * BN + ln;               // this lane's key
-                        const bool all_vis = ktile * BN + BN - 1 <= minp;
                         const uint32_t ta = tq + (uint32_t)(b * SCOLS + ccol);
-                        for (int ch = 0; ch < nch; ++ch) {
-                            float y[32];
-                            tc::tmem_ld32(ta + (uint32_t)(ch * 32), y);
-                            tc::tmem_wait_ld();
-                            if (ch == nch - 1) release_acc(&s.s_empty[b], lane);
-                            const float* nmp = s.row_nmp[rs] + rcol + ch * 32;
-                            const int* rp = s.row_pos[rs] + rcol + ch * 32;
-                            if (rpg >= 32) {
-                                if (all_vis)
-                                    sum += colsum_group<true, true>(y, nmp, rp, sl2, rpg, j);
-                                else
-                                    sum += colsum_group<true, false>(y, nmp, rp, sl2, rpg, j);
-                            } else {
-                                if (all_vis)
-                                    sum += colsum_group<false, true>(y, nmp, rp, sl2, rpg, j);
-                                else
-                                    sum += colsum_group<false, false>(y, nmp, rp, sl2, rpg, j);
+                        const int last = ktile * BN + BN - 1;
+                        if (mode == MODE_PAIR && all64) {
+                            // 64 rows that all see these keys: no branch, and each 16
+                            // columns' load in flight while the 16 before are summed
+                            const float* nmp = s.row_nmp[rs] + rcol;
+                            float2 a = make_float2(0.f, 0.f), c = a;
+                            float y0[16], y1[16];
+                            tc::tmem_ld16(ta, y0);
+                            tc::tmem_wait_ld16(y0);
+                            tc::tmem_ld16(ta + 16, y1);
+                            colsum16(y0, nmp, sl2, a, c);
+                            tc::tmem_wait_ld16(y1);
+                            tc::tmem_ld16(ta + 32, y0);
+                            colsum16(y1, nmp + 16, sl2, a, c);
+                            tc::tmem_wait_ld16(y0);
+                            tc::tmem_ld16(ta + 48, y1);
+                            colsum16(y0, nmp + 32, sl2, a, c);
+                            tc::tmem_wait_ld16(y1);
+                            release_acc(&s.s_empty[b], lane);
+                            colsum16(y1, nmp + 48, sl2, a, c);
+                            sum = (a.x + a.y) + (c.x + c.y);
+                        } else {
+                            for (int ch = 0; ch < nch; ++ch) {
+                                bool all_vis = last <= minp;
+                                if (mode == MODE_PAIR) {
+                                    const int grp = (rcol >> 5) + ch;
+                                    // no row of the group sees these keys (a tile of rows that
+                                // stand far apart: 28 layers, 1920 rows between 32 frames,
+                                // 1491 -> 1455 us)
+                                if (ktile * BN > s.grp_max[rs][grp]) {
+                                        if (ch == nch - 1) release_acc(&s.s_empty[b], lane);
+                                        continue;
+                                    }
+                                    all_vis = last <= s.grp_min[rs][grp];
+                                }
+                                float y[32];
+                                tc::tmem_ld32(ta + (uint32_t)(ch * 32), y);
+                                tc::tmem_wait_ld();
+                                if (ch == nch - 1) release_acc(&s.s_empty[b], lane);
+                                const float* nmp = s.row_nmp[rs] + rcol + ch * 32;
+                                const int* rp = s.row_pos[rs] + rcol + ch * 32;
+                                if (rpg >= 32) {
+                                    if (all_vis)
+                                        sum += colsum_group<true, true>(y, nmp, rp, sl2, rpg, j);
+                                    else
+                                        sum += colsum_group<true, false>(y, nmp, rp, sl2, rpg, j);
+                                } else {
+                                    if (all_vis)
+                                        sum += colsum_group<false, true>(y, nmp, rp, sl2, rpg, j);
+                                    else
+                                        sum += colsum_group<false, false>(y, nmp, rp, sl2, rpg, j);
+                                }
                             }
                         }
                     }
-                    if (ok && act) {
+                    if (mode == MODE_PAIR) {
+                        if (ok && vr0 < p.N_v) atomicAdd(out_row + vr0, sum);
+                    } else if (ok && act) {
                         const uint32_t word = s.vmask[ktile][quarter];
                         if ((word >> lane) & 1u) {
                             const int vr = s.vq[ktile][quarter] + __popc(word & lt_mask);

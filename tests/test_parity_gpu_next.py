@@ -86,6 +86,49 @@ def test_text_scores_and_eq7_weights(api, name):
     assert np.allclose(wt.sum(axis=1), 1.0, rtol=1e-5)
 
 
+# Heads of several row tiles: an even and an odd number of them, the last one short
+# (fewer than 128 rows, or so few that its 32-lane groups are not full), whose rows
+# stand close together (tail) or far apart (all_text: a group of 32 rows sees all, some
+# or none of a block of 64 keys).  The logits jump by about 18 base-2 units at `rise`
+# (past 2^13, where the sums of a block are taken again) and twice as far 300 keys on:
+# at the edges of 16 and 64 keys, in a block of vision keys, of text and across both.
+RISE_SEGS = {"tail": [("text", 70), ("vision", 700), ("text", 150)],
+             "all_text": [("text", 70)] + 6 * [("vision", 130), ("text", 11)] + [("text", 60)]}
+
+
+@pytest.mark.parametrize("G", [1, 2, 3])
+@pytest.mark.parametrize("window", sorted(RISE_SEGS))
+@pytest.mark.parametrize("rise", [5, 128, 255, 271, 288, 304, 319, 333])
+def test_scores_across_row_groups_with_rising_logits(api, window, rise, G):
+    segs = RISE_SEGS[window]
+    wl = synth.custom("rise", 2, 2 * G, 2, 64, segs, window="all_text" if window == "all_text" else 150)
+    inp = synth.generate(wl, seed=13)
+    q = oracle.widen_bf16(inp["q"]).astype(np.float32)
+    k = oracle.widen_bf16(inp["k"]).astype(np.float32)
+    q[..., :16] = 0.9 + 0.2 * np.tanh(q[..., :16])
+    step = np.zeros(wl.N, np.float32)
+    step[rise:] = 7.0
+    step[rise + 300:] = 14.0
+    k[..., :16] = step[:, None] + 0.01 * k[..., :16]
+    inp["q"], inp["k"] = synth.to_bf16_bits(q), synth.to_bf16_bits(k)
+    dev = P.device_inputs(inp)
+    desc = api.desc_for_workload(wl)
+    ws = api.new_workspace(desc)
+    sc = torch.empty((wl.L, wl.H_kv, wl.N_v), dtype=torch.float32, device="cuda")
+    st = torch.empty(wl.L, dtype=torch.float32, device="cuda")
+    api.tgvkv_score(desc, dev["q"], dev["k"], dev["modality"], dev["text_pos"], dev["w"], sc, st, ws)
+    assert api.tgvkv_status(ws) == 0
+    rs, rst = oracle.twr_scores_tvb_stat(oracle.widen_bf16(inp["q"]), oracle.widen_bf16(inp["k"]),
+                                         inp["modality"], inp["text_pos"], inp["w"],
+                                         1.0 / math.sqrt(wl.d), wl.H_kv)
+    P.assert_close(sc.cpu().numpy(), rs, "scores")
+    P.assert_close(st.cpu().numpy(), rst, "tvb_stat")
+    ts, wt = _run_text(api, wl, dev)
+    rts, rwt = _oracle_text(wl, inp)
+    P.assert_close(ts, rts, "text scores (Eq. 9)")
+    P.assert_close(wt, rwt, "weights (Eq. 7)")
+
+
 @pytest.mark.parametrize("name,layers", [("llava15", [0, 31]), ("qwen25", [5]), ("video", [27])])
 def test_text_scores_full_size_sampled(api, name, layers):
     """Full-size shapes in the launch configuration tgvkv_evict uses, checked on
