@@ -209,35 +209,49 @@ __device__ __forceinline__ bool next_step(const Item& it, int mode, int pass, in
     return true;
 }
 
-// Sum over the valid rows of one 32-row group of 2^(y_i sl2 + nmp_i), with the
-// causal mask j <= pos_i.  FULL: all 32 rows exist; ALL_VIS: every row sees
-// key j (no mask; a template argument, so that the unrolled loop has no
-// branch on it).
-template <bool FULL, bool ALL_VIS>
-__device__ __forceinline__ float colsum_group(const float (&y)[32], const float* nmp,
-                                              const int* pos, float sl2, int rpg, int j) {
+// Sum over the rows of one 32-row group of 2^(y_i sl2 + nmp_i), with the causal
+// mask j <= pos_i.  ROWS: the rpg rows that exist, rounded up to 4; ALL_VIS: every
+// row sees key j (both template arguments, so that the unrolled loop has no branch:
+// with one every four rows, 32 layers x 32 heads x 96 rows x 3008 keys took 384 us
+// instead of 380, 24 layers of 64-dim heads of 6 row tiles 45.8 instead of 39.9).
+template <int ROWS, bool ALL_VIS>
+__device__ __forceinline__ float colsum_rows(const float (&y)[32], const float* nmp, const int* pos,
+                                             float sl2, int j) {
     const float2 s2 = make_float2(sl2, sl2);
     float2 a = make_float2(0.f, 0.f), b = a;
 #pragma unroll
-    for (int i = 0; i < 32; i += 4) {
-        if (FULL || i < rpg) {
-            const float4 n4 = *reinterpret_cast<const float4*>(nmp + i);
-            const float2 t0 = fma2(make_float2(y[i], y[i + 1]), s2, make_float2(n4.x, n4.y));
-            const float2 t1 = fma2(make_float2(y[i + 2], y[i + 3]), s2, make_float2(n4.z, n4.w));
-            float2 e0 = make_float2(fast_exp2(t0.x), fast_exp2(t0.y));
-            float2 e1 = make_float2(fast_exp2(t1.x), fast_exp2(t1.y));
-            if (!ALL_VIS) {
-                const int4 p4 = *reinterpret_cast<const int4*>(pos + i);
-                if (j > p4.x) e0.x = 0.f;
-                if (j > p4.y) e0.y = 0.f;
-                if (j > p4.z) e1.x = 0.f;
-                if (j > p4.w) e1.y = 0.f;
-            }
-            a = add2(a, e0);
-            b = add2(b, e1);
+    for (int i = 0; i < ROWS; i += 4) {
+        const float4 n4 = *reinterpret_cast<const float4*>(nmp + i);
+        const float2 t0 = fma2(make_float2(y[i], y[i + 1]), s2, make_float2(n4.x, n4.y));
+        const float2 t1 = fma2(make_float2(y[i + 2], y[i + 3]), s2, make_float2(n4.z, n4.w));
+        float2 e0 = make_float2(fast_exp2(t0.x), fast_exp2(t0.y));
+        float2 e1 = make_float2(fast_exp2(t1.x), fast_exp2(t1.y));
+        if (!ALL_VIS) {
+            const int4 p4 = *reinterpret_cast<const int4*>(pos + i);
+            if (j > p4.x) e0.x = 0.f;
+            if (j > p4.y) e0.y = 0.f;
+            if (j > p4.z) e1.x = 0.f;
+            if (j > p4.w) e1.y = 0.f;
         }
+        a = add2(a, e0);
+        b = add2(b, e1);
     }
     return (a.x + a.y) + (b.x + b.y);
+}
+
+template <bool ALL_VIS>
+__device__ __forceinline__ float colsum_group(const float (&y)[32], const float* nmp, const int* pos,
+                                              float sl2, int rpg, int j) {
+    if (rpg > 28) return colsum_rows<32, ALL_VIS>(y, nmp, pos, sl2, j);
+    switch ((rpg + 3) >> 2) {
+        case 7: return colsum_rows<28, ALL_VIS>(y, nmp, pos, sl2, j);
+        case 6: return colsum_rows<24, ALL_VIS>(y, nmp, pos, sl2, j);
+        case 5: return colsum_rows<20, ALL_VIS>(y, nmp, pos, sl2, j);
+        case 4: return colsum_rows<16, ALL_VIS>(y, nmp, pos, sl2, j);
+        case 3: return colsum_rows<12, ALL_VIS>(y, nmp, pos, sl2, j);
+        case 2: return colsum_rows<8, ALL_VIS>(y, nmp, pos, sl2, j);
+        default: return colsum_rows<4, ALL_VIS>(y, nmp, pos, sl2, j);
+    }
 }
 
 // a + c += the sum over 16 rows of 2^(y_i sl2 + nmp_i): colsum_group of rows that
@@ -1010,17 +1024,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                                 if (ch == nch - 1) release_acc(&s.s_empty[b], lane);
                                 const float* nmp = s.row_nmp[rs] + rcol + ch * 32;
                                 const int* rp = s.row_pos[rs] + rcol + ch * 32;
-                                if (rpg >= 32) {
-                                    if (all_vis)
-                                        sum += colsum_group<true, true>(y, nmp, rp, sl2, rpg, j);
-                                    else
-                                        sum += colsum_group<true, false>(y, nmp, rp, sl2, rpg, j);
-                                } else {
-                                    if (all_vis)
-                                        sum += colsum_group<false, true>(y, nmp, rp, sl2, rpg, j);
-                                    else
-                                        sum += colsum_group<false, false>(y, nmp, rp, sl2, rpg, j);
-                                }
+                                if (all_vis)
+                                    sum += colsum_group<true>(y, nmp, rp, sl2, rpg, j);
+                                else
+                                    sum += colsum_group<false>(y, nmp, rp, sl2, rpg, j);
                             }
                         }
                     }

@@ -86,6 +86,33 @@ def test_text_scores_and_eq7_weights(api, name):
     assert np.allclose(wt.sum(axis=1), 1.0, rtol=1e-5)
 
 
+# Every number of rows in a 32-lane group (the column sums are unrolled for it in steps
+# of four): n_win rows of one head, two heads to a tile up to 64 and one above; G = 3
+# makes several tiles of the larger ones.  Half of the rows stand before the second
+# image, so that key tiles hold keys that all, some or none of them see.
+@pytest.mark.parametrize("G", [1, 3])
+@pytest.mark.parametrize("n_win", [2, 5, 9, 16, 18, 25, 33, 41, 48, 55, 64, 65, 72, 77, 81, 95, 100,
+                                   109, 115, 128])
+def test_scores_row_counts(api, n_win, G):
+    a = n_win // 2
+    wl = synth.custom("rows", 1, 3 * G, 3, 64, [("text", 6), ("vision", 140), ("text", a),
+                                                ("vision", 195), ("text", n_win - a)],
+                      window=n_win, weights="dirichlet")
+    inp = synth.generate(wl, seed=14)
+    dev = P.device_inputs(inp)
+    desc = api.desc_for_workload(wl)
+    ws = api.new_workspace(desc)
+    sc = torch.empty((wl.L, wl.H_kv, wl.N_v), dtype=torch.float32, device="cuda")
+    st = torch.empty(wl.L, dtype=torch.float32, device="cuda")
+    api.tgvkv_score(desc, dev["q"], dev["k"], dev["modality"], dev["text_pos"], dev["w"], sc, st, ws)
+    assert api.tgvkv_status(ws) == 0
+    rs, rst = oracle.twr_scores_tvb_stat(oracle.widen_bf16(inp["q"]), oracle.widen_bf16(inp["k"]),
+                                         inp["modality"], inp["text_pos"], inp["w"],
+                                         1.0 / math.sqrt(wl.d), wl.H_kv)
+    P.assert_close(sc.cpu().numpy(), rs, "scores")
+    P.assert_close(st.cpu().numpy(), rst, "tvb_stat")
+
+
 # Heads of several row tiles: an even and an odd number of them, the last one short
 # (fewer than 128 rows, or so few that its 32-lane groups are not full), whose rows
 # stand close together (tail) or far apart (all_text: a group of 32 rows sees all, some
