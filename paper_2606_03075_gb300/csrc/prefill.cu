@@ -186,10 +186,14 @@ __device__ __forceinline__ void mask_word(float (&x)[32], int lim) {
 }
 
 // A row's 128 logits of a score tile (TMEM columns from ts) as 2^(x sl2 - m),
-// packed in pk in bf16 pairs; z: their fp32 sum, v: the part of it in the 32-key
-// words that are all vision (bits in vw, the same for every lane of the warp).
-// lim: the last visible key (>= 127: all).  One branch-free block: the words'
-// latencies overlap, and both kinds of warps run the same code.
+// packed in pk in bf16 pairs; z: their fp32 sum, v: the part of it at the vision
+// keys (bits in vw, the same for every lane of the warp): whole 32-key words, or
+// MIXED, for tiles with a word of both kinds, key by key.  lim: the last visible
+// key (>= 127: all).  One branch-free block: the words' latencies overlap, and
+// warps with and without a query row run the same code.  (The mixed words' logits
+// read and exponentiated once more instead, before P is handed on: 10.77 ms for 28
+// layers of N = 8704 whose query rows stand between 32 frames, 9.75 so.)
+template <bool MIXED>
 __device__ __forceinline__ void exp_row(uint32_t ts, float sl2, float m, int lim,
                                         const uint32_t (&vw)[4], uint32_t (&pk)[64], float& z,
                                         float& v) {
@@ -206,7 +210,7 @@ __device__ __forceinline__ void exp_row(uint32_t ts, float sl2, float m, int lim
     v = 0.f;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-        float2 za = make_float2(0.f, 0.f), zb = za;
+        float2 za = make_float2(0.f, 0.f), zb = za, va = za, vb = za;
 #pragma unroll
         for (int c = 0; c < 32; c += 4) {
             const float2 t0 = fma2(make_float2(x[w][c], x[w][c + 1]), s2, n2);
@@ -217,37 +221,20 @@ __device__ __forceinline__ void exp_row(uint32_t ts, float sl2, float m, int lim
             pk[16 * w + c / 2 + 1] = pack_bf16(e1.x, e1.y);
             za = add2(za, e0);
             zb = add2(zb, e1);
+            if (MIXED) {
+                if ((vw[w] >> c) & 1u) va.x += e0.x;
+                if ((vw[w] >> c) & 2u) va.y += e0.y;
+                if ((vw[w] >> c) & 4u) vb.x += e1.x;
+                if ((vw[w] >> c) & 8u) vb.y += e1.y;
+            }
         }
         const float zw = (za.x + za.y) + (zb.x + zb.y);
         z += zw;
-        v += vw[w] == ~0u ? zw : 0.f;
+        if (MIXED)
+            v += (va.x + va.y) + (vb.x + vb.y);
+        else
+            v += vw[w] != 0u ? zw : 0.f;
     }
-}
-
-// The vision part of the words that are neither all vision nor all text, from
-// the logits again (they are still in tensor memory): a rolled loop, run at the
-// borders between text and vision only.
-__device__ __forceinline__ float mixed_words(uint32_t ts, float sl2, float m, int lim,
-                                             const uint32_t (&vw)[4]) {
-    float v = 0.f;
-#pragma unroll 1
-    for (int w = 0; w < 4; ++w) {
-        const uint32_t bits = w == 0 ? vw[0] : w == 1 ? vw[1] : w == 2 ? vw[2] : vw[3];
-        if (bits == 0u || bits == ~0u) continue;
-        float x[32];
-        tc::tmem_ld32(ts + (uint32_t)(32 * w), x);
-        tc::tmem_wait_ld();
-        if (!__all_sync(~0u, lim >= 127)) mask_word(x, lim - 32 * w);
-        float2 va = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-            const float2 t = fma2(make_float2(x[c], x[c + 1]), make_float2(sl2, sl2), make_float2(-m, -m));
-            va = add2(va, make_float2((bits >> c) & 1u ? fast_exp2(t.x) : 0.f,
-                                      (bits >> (c + 1)) & 1u ? fast_exp2(t.y) : 0.f));
-        }
-        v += va.x + va.y;
-    }
-    return v;
 }
 
 // Three-input maximum (PTX max.f32 with three sources).
@@ -397,6 +384,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                     vw[2] = u.z;
                     vw[3] = u.w;
                 }
+                const bool mixed = vw[0] + 1u > 1u || vw[1] + 1u > 1u || vw[2] + 1u > 1u || vw[3] + 1u > 1u;
                 // the logits of tile st of this stream: its own S, or S 0 and 1 in turn
                 const int sb = SOLO ? st & 1 : w;
                 const uint32_t ts = tl + (uint32_t)(sb * PN);
@@ -448,14 +436,17 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                             tc::tmem_wait_st();
                         }
                     }
-                    exp_row(ts, sl2, m, lim, vw, pk, z, v);
+                    if (mixed)
+                        exp_row<true>(ts, sl2, m, lim, vw, pk, z, v);
+                    else
+                        exp_row<false>(ts, sl2, m, lim, vw, pk, z, v);
                     if (again || __all_sync(~0u, z <= kTermLimit)) break;
                     again = true;
                 }
                 if (!ok) break;
                 lsum += z;
                 // (lanes without a query row sum a vision mass that is never written)
-                if (want_v) vsum += v + mixed_words(ts, sl2, m, lim, vw);
+                vsum += v;
                 tc::tmem_st32u(ts, *reinterpret_cast<const uint32_t(*)[32]>(pk));
                 tc::tmem_st32u(ts + 32u, *reinterpret_cast<const uint32_t(*)[32]>(pk + 32));
                 tc::tmem_wait_st();
