@@ -957,12 +957,14 @@ cudaError_t launch_prefill(const Problem& p, const uint16_t* q, const uint16_t* 
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + lay.status);
     const int sms = device_sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;
-    // Up to three row tiles per SM the pairs leave SMs idle or end unevenly, and a
+    // Up to four row tiles per SM the pairs leave SMs idle or end unevenly, and a
     // pair's step is no shorter for having the SM's neighbours idle: one head pair of
     // 8000 keys 68 us solo, 111 us in pairs (d = 128), 14 heads of 2833 keys 46 / 51,
-    // 32 heads of 858 keys 25 / 30; above, the pairs' shared K and V tiles win (56 heads
-    // of 1685 keys, 5 tiles per SM: 142 / 120 us).
-    const bool solo = (long long)p.L * p.H_q * ((p.N + PM - 1) / PM) <= 3ll * sms;
+    // 32 heads of 858 keys 25 / 30, 28 heads of 2500 keys (3.7 tiles per SM, d = 64) 41 /
+    // 47; above, the pairs' shared K and V tiles win (56 heads of 1685 keys, 5 tiles per
+    // SM: 142 / 120 us).  One tile per head makes no pair: 1024 heads of 100 keys 35 / 39.
+    const int n_qt = (p.N + PM - 1) / PM;
+    const bool solo = n_qt == 1 || (long long)p.L * p.H_q * n_qt <= 4ll * sms;
     const auto launch = p.d == 64 ? (solo ? launch_prefill_d<64, true> : launch_prefill_d<64, false>)
                                   : (solo ? launch_prefill_d<128, true> : launch_prefill_d<128, false>);
     return launch(p, q, k, v, modality, text_pos, o, q_text, row_stats, work_counter, status, sms,

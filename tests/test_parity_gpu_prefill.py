@@ -433,7 +433,7 @@ EDGES = [(1, 1, 64), (31, 4, 128), (128, 1, 128), (129, 2, 64), (256, 1, 64), (2
 
 
 def _layers(form, heads, n):
-    return 2 if form == "few" else -(-600 // (heads * -(-n // 128)))
+    return 2 if form == "few" else -(-700 // (heads * -(-n // 128)))
 
 
 @pytest.mark.parametrize("form", ["few", "many"])
