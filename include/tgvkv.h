@@ -345,8 +345,9 @@ int tgvkv_evict_launches(const tgvkv_desc* desc);
  * TGVKV_STATUS_INDEX (results then undefined).  capacity_rows < 0 is
  * rejected.  The rows of other sets
  * next to a set's own may be read and are masked: they must be finite.
- * Two kernels: the row streams, then (launched as a programmatic dependent)
- * the merge of the sets they split; the workspace holds the streams' partial
+ * Two kernels: the row streams, then the merge of the sets they split (both
+ * launched as programmatic dependents: they may be scheduled while the kernel
+ * before them on the stream ends, and wait for it on the device); the workspace holds the streams' partial
  * results (tgvkv_workspace_size covers them). */
 int tgvkv_decode(const tgvkv_desc* desc, const uint16_t* q, const uint16_t* k_rows,
                  const uint16_t* v_rows, int64_t capacity_rows, const int64_t* offsets,

@@ -23,10 +23,10 @@
 //               16 bits (a plain bf16 P would move an output by ~1e-3).
 // The softmax is online, in base 2.  A set that one stream covers whole is
 // written out directly; a set split over several streams leaves one partial
-// (m, l, O) per stream, and a second kernel, launched as a programmatic
-// dependent of the first (its launch overlaps the first kernel's tail), merges
-// them: one warp per (set, query head), the partials in stream order, so the
-// result does not depend on timing.  The second kernel also checks the CSR
+// (m, l, O) per stream, and a second kernel merges them, one warp or sixteen per
+// (set, query head), the partials in stream order, so the result does not depend
+// on timing.  Each kernel is a programmatic dependent of the one before it, so
+// that its launch overlaps that kernel's tail.  The second kernel also checks the CSR
 // and writes 0 for empty sets.  Groups of more than 8 query heads take
 // several passes (blockIdx.y), each over all rows.
 #include <cuda_bf16.h>
