@@ -95,7 +95,7 @@ extern "C" {
 #define TGVKV_STATUS_BUDGET       0x04u /* a layer budget outside [0, N_v] reached select */
 #define TGVKV_STATUS_INDEX        0x08u /* compact: an index outside [0, N), decreasing offsets, or a CSR larger than the output; decode: a CSR outside its rows */
 #define TGVKV_STATUS_COUNT        0x10u /* a retained set did not hold N_t + b_l rows */
-#define TGVKV_STATUS_TIMEOUT      0x20u /* a bounded on-chip wait gave up */
+#define TGVKV_STATUS_TIMEOUT      0x20u /* a bounded on-chip wait gave up, or the workspace's work counters were not zero (zero it again) */
 #define TGVKV_STATUS_WEIGHT       0x40u /* a text weight is negative or not finite */
 
 /* ---- modes ------------------------------------------------------------ */
@@ -357,10 +357,18 @@ int tgvkv_decode(const tgvkv_desc* desc, const uint16_t* q, const uint16_t* k_ro
 int tgvkv_decode_launches(const tgvkv_desc* desc);
 
 /* Zero `workspace` (asynchronously on `stream`).  Needed once after the
- * workspace is allocated: the calls leave their completion counters at zero
- * for the next call.  Zero it again after a call whose tgvkv_status reported
+ * workspace is allocated: the calls leave their counters at zero for the next
+ * call.  Zero it again after a call whose tgvkv_status reported
  * TGVKV_STATUS_TIMEOUT, and never share one workspace between calls that may
- * overlap on the GPU. */
+ * overlap on the GPU.
+ * One workspace may serve calls with several descriptors, one after another,
+ * if it has the largest of their sizes.  Its first 256 bytes (the status word
+ * and the work counters) are the same for all of them, which is all that
+ * tgvkv_prefill, tgvkv_decode, tgvkv_budget, the selections and tgvkv_compact
+ * need.  tgvkv_score, tgvkv_text_scores and tgvkv_evict also keep one completion
+ * counter per KV head behind them, where a descriptor with fewer heads has its
+ * scratch: zero the workspace before such a call when a call with another
+ * L * H_kv has used it since. */
 int tgvkv_workspace_init(const tgvkv_desc* desc, void* workspace, void* stream);
 
 /* Synchronise `stream`, then read and clear the device status word kept in

@@ -46,8 +46,10 @@ bool needs_text_pass(const Problem& p) {
 WsLayout layout_of(const Problem& p) {
     WsLayout w;
     size_t o = 0;
-    w.status = o;      o += round_up(sizeof(uint32_t));
-    w.tickets = o;     o += round_up(sizeof(uint32_t) * ticket_words(p));
+    w.status = kWsStatus;
+    w.counters = kWsCounters;
+    o += kWsFixed;
+    w.tickets = o;     o += round_up(sizeof(uint32_t) * (size_t)p.L * p.H_kv);
     w.stat_part = o;   o += round_up(sizeof(float) * (size_t)p.L * p.H_kv * (p.T > 0 ? p.T : 1));
     w.stat_head = o;   o += round_up(sizeof(float) * (size_t)p.L * p.H_kv);
     w.score_part = o;
@@ -654,11 +656,11 @@ extern "C" int tgvkv_score_noalloc(const tgvkv_desc* desc, const uint16_t* q_tex
     rc = check_score_args(p, q_text, k, modality, text_pos, w, scores, tvb_stat, scratch);
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the status word and the completion counters start at zero for every call
-    cudaError_t e = cudaMemsetAsync(static_cast<char*>(scratch) + lay.status, 0, sizeof(uint32_t), st);
+    // the status word and the counters start at zero for every call
+    cudaError_t e = cudaMemsetAsync(static_cast<char*>(scratch) + lay.status, 0, kWsFixed, st);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(static_cast<char*>(scratch) + lay.tickets, 0,
-                            sizeof(uint32_t) * ticket_words(p), st);
+                            sizeof(uint32_t) * (size_t)p.L * p.H_kv, st);
     if (e != cudaSuccess) return cuda_fail(e, "static scratch clear");
     rc = do_score(p, q_text, k, modality, text_pos, w, scores, tvb_stat, scratch, st);
     return rc ? rc : ok();

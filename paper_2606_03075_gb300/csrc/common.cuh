@@ -51,8 +51,11 @@ __host__ __device__ inline bool is_sink(const Problem& p, int j) {
 
 // Workspace layout (byte offsets into the caller's buffer).
 struct WsLayout {
+    // at the same place for every descriptor (kWsStatus, kWsCounters):
     size_t status;      // uint32 status word
-    size_t tickets;     // uint32 [ticket_words]: completion counters (heads), kernel counters
+    size_t counters;    // uint32 [kWsCounterWords]: the kernels' work counters
+    // the places below follow from the descriptor:
+    size_t tickets;     // uint32 [L*H_kv]: the score kernel's completion counters
     size_t stat_part;   // float [L*H_kv*T]: TV mass of one row tile
     size_t stat_head;   // float [L*H_kv]: TV mass of one KV head
     size_t score_part;  // float [L*H_kv*T*max(N_v,N_t)]: scores of one row tile (T > 1)
@@ -73,11 +76,22 @@ __host__ __device__ inline int score_pairs(const Problem& p) {
     return p.T >= 2 ? (p.T + 1) / 2 : 1;
 }
 
-// Counters at the start of the workspace: one per KV head, then the score
-// kernel's work counter, the count of CTAs that ran out of work, and the count
-// of CTAs that finished.
-__host__ __device__ inline size_t ticket_words(const Problem& p) {
-    return (size_t)p.L * p.H_kv + 3;
+// The first 256 bytes of a workspace are the same for every descriptor: the status
+// word, and the work counters of the score and prefill kernels (the next item, the
+// count of CTAs that ran out of work, the count of CTAs that finished).  No other
+// call's scratch ever lies over them, whatever descriptor it had.
+constexpr size_t kWsStatus = 0, kWsCounters = 64, kWsFixed = 256;
+constexpr int kWsCounterWords = 3;
+
+// A claim of work items: `first` items are taken without a claim.  A counter that
+// was not zero when the launch began can give any value: the comparison is
+// unsigned, so that an item is always in range, and a value above what a launch of
+// n items reaches (it claims n times) reports the counter.
+__device__ __forceinline__ uint32_t claim_item(uint32_t* counter, uint32_t first, int n,
+                                               uint32_t* status) {
+    const uint32_t id = first + atomicAdd(counter, 1u);
+    if (id >= first + (uint32_t)n) atomicOr(status, TGVKV_STATUS_TIMEOUT);
+    return id;
 }
 
 constexpr int kMaxN = 32768;     // key positions per head (the per-CTA tile maps)

@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             bool ok = true;
             // the first item of CTA c is item c (grid <= items); later ones are claimed,
             // an item ahead, so that the claim's latency hides behind the item's loads
-            int id = (int)blockIdx.x;
+            uint32_t id = blockIdx.x;
             for (int n = 0; ok; ++n) {
                 const int islot = n % PIQ;
                 if (!tc::mbar_wait(&s.it_empty[islot], ((n / PIQ) & 1) ^ 1, abort_flag)) {
@@ -604,22 +604,17 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 PItem itm;
                 itm.hi = -1;
                 itm.lhq = 0;
-                if (id < n_items) itm = prefill_item(p, n_qt, SOLO ? 1 : 2, batch, id);
+                const bool more = id < (uint32_t)n_items;
+                if (more) itm = prefill_item(p, n_qt, SOLO ? 1 : 2, batch, (int)id);
                 s.item_hi[islot] = itm.hi;
                 s.item_lhq[islot] = itm.lhq;
                 tc::mbar_arrive(&s.it_full[islot]);
-                if (id >= n_items) {
+                if (!more) {
                     if (SOLO && g > 1) load(&tmap_v, v_tile[0], v_row[0]);
                     if (SOLO && ok && g > 0) load(&tmap_v, v_tile[1], v_row[1]);
-                    // the last CTA to run out of work re-arms the counter for the next launch
-                    if (atomicAdd(done_counter, 1u) == gridDim.x - 1) {
-                        atomicExch(work_counter, 0u);
-                        atomicExch(done_counter, 0u);
-                        __threadfence();
-                    }
                     break;
                 }
-                const int next = (int)gridDim.x + (int)atomicAdd(work_counter, 1u);
+                const uint32_t next = claim_item(work_counter, gridDim.x, n_items, status);
                 const int q_row = itm.lhq * p.N, kv_row = (itm.lhq / p.G) * p.N;
                 auto load_q = [&](int slot, int t) {
                     int& uses = slot == 0 ? q0 : q1;
@@ -664,6 +659,13 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             if (!ok) {
                 s.abort_flag = 1;
                 raise_status(status, TGVKV_STATUS_TIMEOUT);
+            }
+            // the last CTA to run out of work (or to give up) re-arms the counters for the
+            // next launch
+            if (atomicAdd(done_counter, 1u) == gridDim.x - 1) {
+                atomicExch(work_counter, 0u);
+                atomicExch(done_counter, 0u);
+                __threadfence();
             }
             // every copy this CTA issued has landed before it may exit
             if (q0 > 0) tc::mbar_wait(&s.q_full[0], (q0 - 1) & 1, &s.never);
@@ -953,7 +955,7 @@ cudaError_t launch_prefill(const Problem& p, const uint16_t* q, const uint16_t* 
                            const uint16_t* v, const uint8_t* modality, const int32_t* text_pos,
                            uint16_t* o, uint16_t* q_text, float* row_stats, char* ws,
                            const WsLayout& lay, cudaStream_t stream) {
-    uint32_t* work_counter = reinterpret_cast<uint32_t*>(ws + lay.tickets) + (size_t)p.L * p.H_kv;
+    uint32_t* work_counter = reinterpret_cast<uint32_t*>(ws + lay.counters);
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + lay.status);
     const int sms = device_sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;

@@ -318,7 +318,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 float* __restrict__ scores, float* __restrict__ tvb_stat,
                 float* __restrict__ score_part, float* __restrict__ stat_part,
                 float* __restrict__ stat_head, uint32_t* __restrict__ tickets,
-                uint32_t* __restrict__ status, long long budget_total, int32_t* __restrict__ budgets) {
+                uint32_t* __restrict__ work_counter, uint32_t* __restrict__ status,
+                long long budget_total, int32_t* __restrict__ budgets) {
     float* row_stats = p.row_stats;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -333,7 +334,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float sl2 = p.scale_log2;
     const int LH = p.L * p.H_kv;
-    uint32_t* work_counter = tickets + LH;
     uint32_t* done_counter = work_counter + 1;
     uint32_t* exit_counter = work_counter + 2;
 
@@ -451,10 +451,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 break;
             }
             // the first item of CTA c is item c (grid <= items); later ones are claimed
-            const int id = n == 0 ? (int)blockIdx.x : (int)gridDim.x + (int)atomicAdd(work_counter, 1u);
-            s.item_q[slot] = id < n_items ? id : -1;
+            const uint32_t claim =
+                n == 0 ? blockIdx.x : claim_item(work_counter, gridDim.x, n_items, status);
+            const int id = claim < (uint32_t)n_items ? (int)claim : -1;
+            s.item_q[slot] = id;
             tc::mbar_arrive(&s.it_full[slot]);
-            if (id >= n_items) {
+            if (id < 0) {
                 // the last CTA to run out of work re-arms the counter for the next launch
                 if (atomicAdd(done_counter, 1u) == gridDim.x - 1) {
                     *work_counter = 0u;
@@ -1226,6 +1228,7 @@ cudaError_t launch_mode(const CUtensorMap& mq, const CUtensorMap& mk, const Prob
                             reinterpret_cast<float*>(ws + lay.stat_part),
                             reinterpret_cast<float*>(ws + lay.stat_head),
                             reinterpret_cast<uint32_t*>(ws + lay.tickets),
+                            reinterpret_cast<uint32_t*>(ws + lay.counters),
                             reinterpret_cast<uint32_t*>(ws + lay.status), budget_total, budgets);
 }
 

@@ -449,6 +449,35 @@ def test_prefill_tile_edges(api, n, group, d, form):
     _check_prefill(wl, inp, *out, layers=sorted({0, wl.L // 2, wl.L - 1}))
 
 
+@pytest.mark.parametrize("L,n", [(32, 120), (32, 270)])
+def test_prefill_in_a_workspace_of_other_calls(api, L, n):
+    """A model's prefill in the workspace in which its layers decode one by one, over
+    and over: the decode's partial results lie where a descriptor with more KV heads
+    has its per-head counters, and the prefill gives the same bits each time."""
+    wl = synth.custom("shared_ws", L, 16, 8, 64, [("text", 20), ("vision", n - 90), ("text", 70)])
+    inp = synth.generate_prefill(wl, seed=15)
+    dev = P.device_inputs(inp)
+    ref = _run_prefill(api, wl, inp, dev)
+    desc = api.desc_for_workload(wl)
+    one = api.make_desc(1, wl.H_q, wl.H_kv, wl.d, wl.N, wl.N_v, 0)
+    ws = torch.empty(max(api.tgvkv_workspace_size(desc), api.tgvkv_workspace_size(one)),
+                     dtype=torch.uint8, device="cuda")
+    api.tgvkv_workspace_init(desc, ws)
+    q_all = _bf16(inp["q_all"])
+    offsets = torch.arange(wl.H_kv + 1, dtype=torch.int64, device="cuda") * wl.N
+    step = torch.empty((1, wl.H_q, wl.d), dtype=torch.float32, device="cuda")
+    for _ in range(3):
+        got = [torch.full_like(t, float("nan")) for t in ref]
+        api.tgvkv_prefill(desc, q_all, dev["k"], dev["v"], dev["modality"], dev["text_pos"], *got, ws)
+        assert api.tgvkv_status(ws) == 0
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b)
+        for l in range(wl.L):
+            api.tgvkv_decode(one, q_all[l, :, -1].contiguous(), dev["k"][l].view(-1, wl.d),
+                             dev["v"][l].view(-1, wl.d), offsets, step, ws)
+        assert api.tgvkv_status(ws) == 0
+
+
 @pytest.mark.parametrize("form", ["few", "many"])
 @pytest.mark.parametrize("first_rise", [20, 70, 140, 200, 330])
 def test_prefill_rising_logits(api, first_rise, form):
