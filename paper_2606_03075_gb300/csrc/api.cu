@@ -316,7 +316,7 @@ int evict_impl(const tgvkv_desc* desc, const uint16_t* q_text, const uint16_t* k
         if (e != cudaSuccess) return cuda_fail(e, "budget launch");
     }
     e = launch_select_compact(p, scores, text_scores, budgets, modality, offsets, idx, k, v, k_out,
-                              v_out, retained_rows(p, ratio), status, st);
+                              v_out, retained_rows(p, ratio), status, st, score_launches(p) > 0);
     if (e != cudaSuccess) return cuda_fail(e, "select/compact launch");
     return ok();
 }
@@ -479,7 +479,7 @@ int tgvkv_select_compact(const tgvkv_desc* desc, const float* scores, const floa
     const long long cap = std::min((long long)capacity_rows, (long long)p.L * p.H_kv * p.N);
     cudaError_t e = launch_select_compact(p, scores, text_scores, budgets, modality, offsets, idx,
                                           k, v, k_out, v_out, cap, status_of(workspace, lay),
-                                          static_cast<cudaStream_t>(stream));
+                                          static_cast<cudaStream_t>(stream), false);
     return e == cudaSuccess ? ok() : cuda_fail(e, "select/compact launch");
 }
 

@@ -70,12 +70,16 @@ cudaError_t launch_select(const Problem& p, const float* scores, const float* te
 // select + gather fused (tgvkv_evict): one CTA per (layer, KV head) selects
 // its set and gathers its rows; falls back to the separate select and compact
 // kernels when the keys and retained rows of a head do not fit in shared
-// memory.
+// memory.  after_score: the kernel before on the stream is the score kernel, all of
+// whose CTAs waited for the kernel before them first and let this one start then: the modality
+// is then written, and is read before this kernel's own wait.  After any other kernel
+// (a caller's, which may signal early) the wait comes first.
 cudaError_t launch_select_compact(const Problem& p, const float* scores, const float* text_scores,
                                   const int32_t* budgets, const uint8_t* modality,
                                   int64_t* offsets, int32_t* idx, const uint16_t* k,
                                   const uint16_t* v, uint16_t* k_out, uint16_t* v_out,
-                                  long long capacity_rows, uint32_t* status, cudaStream_t stream);
+                                  long long capacity_rows, uint32_t* status, cudaStream_t stream,
+                                  bool after_score);
 
 // Eq. 7 weights from the Eq. 9 text scores (text.cu): weights[l][j] for the
 // query rows, L1-normalised per layer.

@@ -313,8 +313,8 @@ __device__ __forceinline__ void release_acc(uint64_t* bar, int lane) {
 template <int D, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
-                Problem p, int n_items, int n_two, const uint8_t* __restrict__ modality,
-                const int32_t* __restrict__ text_pos, const float* __restrict__ w,
+                Problem p, int n_items, int n_two, const uint8_t* modality,
+                const int32_t* text_pos, const float* w,
                 float* __restrict__ scores, float* __restrict__ tvb_stat,
                 float* __restrict__ score_part, float* __restrict__ stat_part,
                 float* __restrict__ stat_head, uint32_t* __restrict__ tickets,
@@ -338,13 +338,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     uint32_t* exit_counter = work_counter + 2;
 
     // ------------------------------------------------------------ prologue
-    if (blockIdx.x == 0) {
-        for (int i = tid; i < p.n_win; i += NTHREADS) {
-            const int pi = text_pos[i];
-            if (pi < 0 || pi >= p.N || (i > 0 && text_pos[i - 1] >= pi))
-                raise_status(status, TGVKV_STATUS_TEXT_POS);
-        }
-    }
     if (tid == 0) {
         s.abort_flag = 0;
         s.never = 0;
@@ -369,17 +362,38 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         tc::tmem_alloc(&s.tmem_base, TMEM_COLS);
         tc::tmem_relinquish();
     }
+    if (tid == NTHREADS - 1) {
+        tc::tma_prefetch_desc(&tmap_q);
+        tc::tma_prefetch_desc(&tmap_k);
+    }
+    // Launched as a programmatic dependent, this CTA may have started while the kernel
+    // before it runs: one of a caller that signals early and still writes the inputs, or
+    // the select + gather of the previous eviction, which still reads the scores and
+    // budgets.  Every thread waits for it before any input is read (through L2, not the
+    // read-only path) or any result written.  (With the tables, the first loads and MMAs
+    // before the wait, evictions back to back took 16.8 instead of 18.7 us for one layer of
+    // 112 tokens, 86.4 / 90.0 for 1024 heads of 675, 366 / 370 for 1024 heads of 3008; the
+    // first loads ahead of the tables: no difference.)
+    griddep_wait();
+    if (blockIdx.x == 0) {
+        for (int i = tid; i < p.n_win; i += NTHREADS) {
+            const int pi = __ldcg(text_pos + i);
+            if (pi < 0 || pi >= p.N || (i > 0 && __ldcg(text_pos + i - 1) >= pi))
+                raise_status(status, TGVKV_STATUS_TEXT_POS);
+        }
+    }
     const int n_tiles_all = (p.N + BN - 1) / BN;
     // the first row positions are loaded now, so that their latency overlaps
     // the modality loads below
-    const int pos0 = tid < p.R ? text_pos[tid % p.n_win] : -1;
+    const int pos0 = tid < p.R ? __ldcg(text_pos + tid % p.n_win) : -1;
     for (int kt = warp; kt < n_tiles_all; kt += NTHREADS / 32) {
         int cnt = 0;
 #pragma unroll
         for (int wd = 0; wd < 4; ++wd) {
             const int j = kt * BN + wd * 32 + lane;
             // the key set of pass B: vision keys, or text keys (Eq. 9)
-            const unsigned m = __ballot_sync(~0u, j < p.N && (modality[j] != 0) != (p.keys_text != 0));
+            const unsigned m =
+                __ballot_sync(~0u, j < p.N && (__ldcg(modality + j) != 0) != (p.keys_text != 0));
             if (lane == 0) {
                 s.vmask[kt][wd] = m;
                 s.vq[kt][wd] = cnt;              // within the tile, for now
@@ -396,7 +410,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     __syncthreads();
     tc::fence_after_sync();
     for (int r = tid; r < p.R; r += NTHREADS) {
-        const int pos = r == tid ? pos0 : text_pos[r % p.n_win];
+        const int pos = r == tid ? pos0 : __ldcg(text_pos + r % p.n_win);
         if (pos >= 0 && pos < p.N) {
             atomicMax(&s.rt_max[r / BM], pos);
             atomicMin(&s.rt_min[r / BM], pos);
@@ -438,8 +452,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     // Items are claimed from a counter in order, longest first (pair items
     // differ in length); CTA c starts with item c without a claim.
     if (warp == 0 && lane == 0) {
-        tc::tma_prefetch_desc(&tmap_q);
-        tc::tma_prefetch_desc(&tmap_k);
         int it = 0;
         int qn0 = 0, qn1 = 0;     // uses of each Q slot
         bool ok = true;
@@ -641,11 +653,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
     // ------------------------------------------------------------ softmax
     if (warp >= 2 && warp < MMA2_WARP) {
-        // The kernel before (the select + gather of the previous eviction, when it
-        // is one) may still read the scores and budgets this kernel overwrites: the
-        // softmax role, the only one writing global memory before the end, waits
-        // for it.  The loads and MMAs of the first items overlap its end.
-        griddep_wait();
         const int sid = tid - 64;
         const int quarter = warp & 3;
         const int wi = (warp - 2) >> 2;                     // 0..3 within the lane quarter
@@ -694,12 +701,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                 if (has) {
                     const int t_row = mode == MODE_PAIR ? (2 * itm.pidx + rs) * BM : 0;
                     const int wi_row = (t_row + row) % p.n_win;
-                    pos = text_pos[wi_row];
+                    pos = __ldcg(text_pos + wi_row);
                     if (pos < 0 || pos >= p.N) pos = -1;
                     if (p.keys_text) {
                         wr = 1.f;   // Eq. 9: unweighted column sums
                     } else {
-                        wr = w[(long long)Item::pick(itm.l, part) * p.w_stride + wi_row];
+                        wr = __ldcg(w + (long long)Item::pick(itm.l, part) * p.w_stride + wi_row);
                         if (!(wr >= 0.f) || isinf(wr)) {
                             raise_status(status, TGVKV_STATUS_WEIGHT);
                             wr = 0.f;

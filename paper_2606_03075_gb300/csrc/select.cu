@@ -138,7 +138,8 @@ tpr_select_kernel(Problem p, const float* __restrict__ scores, const int32_t* __
                   const uint8_t* __restrict__ modality_g, int64_t* __restrict__ offsets,
                   int32_t* __restrict__ idx, const uint4* __restrict__ k,
                   const uint4* __restrict__ v, uint4* __restrict__ k_out,
-                  uint4* __restrict__ v_out, long long capacity, uint32_t* __restrict__ status) {
+                  uint4* __restrict__ v_out, long long capacity, uint32_t* __restrict__ status,
+                  bool after_score) {
     extern __shared__ __align__(16) unsigned char dyn_raw[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(dyn_raw);  // [N_v]
     int* rows = reinterpret_cast<int*>(keys + p.N_v);       // [N_t + b] (gather form)
@@ -150,9 +151,11 @@ tpr_select_kernel(Problem p, const float* __restrict__ scores, const int32_t* __
     __shared__ int s_kk;
     __shared__ int s_ties;
 
-    // a kernel after this one (the next eviction's score kernel) reads nothing
-    // this one writes: it may be scheduled once every CTA of this grid has begun
+    // a kernel after this one (the next eviction's score kernel, a decode step) touches
+    // global memory only after its own wait: it may be scheduled once every CTA of this
+    // grid has begun
     if (COMPACT) griddep_launch_dependents();
+    if (!after_score) griddep_wait();   // the modality below may still be written
     // fused form: CTA 2h selects head h and gathers its interior rows, CTA
     // 2h + 1 copies its edge rows
     const int lg = COMPACT ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
@@ -161,7 +164,7 @@ tpr_select_kernel(Problem p, const float* __restrict__ scores, const int32_t* __
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ int span_red[64];
 
-    for (int j = tid; j < p.N; j += kThreads) modality[j] = __ldg(modality_g + j);
+    for (int j = tid; j < p.N; j += kThreads) modality[j] = __ldcg(modality_g + j);
     __syncthreads();
     int vlo = 0, vhi = 0;   // edge rows: positions [0, vlo) and [vhi, N)
     if (COMPACT) vision_span_block(modality, p.N, &vlo, &vhi, span_red);
@@ -420,19 +423,21 @@ tpr_select_warp_kernel(Problem p, const float* __restrict__ scores,
                        int64_t* __restrict__ offsets, int32_t* __restrict__ idx,
                        const uint4* __restrict__ k, const uint4* __restrict__ v,
                        uint4* __restrict__ k_out, uint4* __restrict__ v_out,
-                       long long capacity, uint32_t* __restrict__ status) {
+                       long long capacity, uint32_t* __restrict__ status, bool after_score) {
     extern __shared__ __align__(16) unsigned char dyn_raw[];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
-    // a kernel after this one (the next eviction's score kernel) reads nothing
-    // this one writes: it may be scheduled once every CTA of this grid has begun
+    // a kernel after this one (the next eviction's score kernel, a decode step) touches
+    // global memory only after its own wait: it may be scheduled once every CTA of this
+    // grid has begun
     griddep_launch_dependents();
+    if (!after_score) griddep_wait();   // the modality below may still be written
     const size_t mod_bytes = ((size_t)p.N + 15) & ~size_t(15);
     uint8_t* modality = dyn_raw;
     uint32_t* keys = reinterpret_cast<uint32_t*>(dyn_raw + mod_bytes) + (size_t)wid * warp_select_words(p);
     int* hist = reinterpret_cast<int*>(keys + p.N_v);
     int* rows = hist + 256;
-    for (int j = threadIdx.x; j < p.N; j += blockDim.x) modality[j] = __ldg(modality_g + j);
+    for (int j = threadIdx.x; j < p.N; j += blockDim.x) modality[j] = __ldcg(modality_g + j);
     __syncthreads();
     // CTA 2c selects and gathers the interior rows of heads c*nw.., CTA 2c + 1
     // copies their edge rows (positions [0, vlo) and [vhi, N))
@@ -918,7 +923,8 @@ template <int VPR>
 cudaError_t launch_sel_warp(const Problem& p, int nw, const float* scores, const int32_t* budgets,
                             const uint8_t* modality, int64_t* offsets, int32_t* idx,
                             const uint16_t* k, const uint16_t* v, uint16_t* k_out, uint16_t* v_out,
-                            long long capacity, uint32_t* status, cudaStream_t stream) {
+                            long long capacity, uint32_t* status, cudaStream_t stream,
+                            bool after_score) {
     auto kern = tpr_select_warp_kernel<VPR>;
     const size_t smem = (((size_t)p.N + 15) & ~size_t(15)) + sizeof(uint32_t) * warp_select_words(p) * nw;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -928,14 +934,15 @@ cudaError_t launch_sel_warp(const Problem& p, int nw, const float* scores, const
     return launch_dependent(kern, dim3(2 * ((heads + nw - 1) / nw)), dim3(nw * 32), smem, stream, p,
                             scores, budgets, modality, offsets, idx, reinterpret_cast<const uint4*>(k),
                             reinterpret_cast<const uint4*>(v), reinterpret_cast<uint4*>(k_out),
-                            reinterpret_cast<uint4*>(v_out), capacity, status);
+                            reinterpret_cast<uint4*>(v_out), capacity, status, after_score);
 }
 
 template <bool COMPACT, int VPR>
 cudaError_t launch_sel(const Problem& p, const float* scores, const int32_t* budgets,
                        const uint8_t* modality, int64_t* offsets, int32_t* idx,
                        const uint16_t* k, const uint16_t* v, uint16_t* k_out, uint16_t* v_out,
-                       long long capacity, uint32_t* status, cudaStream_t stream) {
+                       long long capacity, uint32_t* status, cudaStream_t stream,
+                       bool after_score) {
     auto kern = tpr_select_kernel<COMPACT, VPR>;
     const size_t smem = select_smem(p, COMPACT);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -945,12 +952,12 @@ cudaError_t launch_sel(const Problem& p, const float* scores, const int32_t* bud
         return launch_dependent(kern, grid, dim3(kThreads), smem, stream, p, scores, budgets, modality,
                                 offsets, idx, reinterpret_cast<const uint4*>(k),
                                 reinterpret_cast<const uint4*>(v), reinterpret_cast<uint4*>(k_out),
-                                reinterpret_cast<uint4*>(v_out), capacity, status);
+                                reinterpret_cast<uint4*>(v_out), capacity, status, after_score);
     kern<<<grid, kThreads, smem, stream>>>(
         p, scores, budgets, modality, offsets, idx,
         reinterpret_cast<const uint4*>(k),
         reinterpret_cast<const uint4*>(v), reinterpret_cast<uint4*>(k_out),
-        reinterpret_cast<uint4*>(v_out), capacity, status);
+        reinterpret_cast<uint4*>(v_out), capacity, status, after_score);
     return cudaGetLastError();
 }
 
@@ -968,7 +975,7 @@ cudaError_t launch_select_cap(const Problem& p, const float* scores, const float
                                              idx, nullptr, nullptr, nullptr, nullptr, capacity,
                                              status, stream);
     return launch_sel<false, 16>(p, scores, budgets, modality, offsets, idx, nullptr, nullptr, nullptr,
-                                 nullptr, capacity, status, stream);
+                                 nullptr, capacity, status, stream, false);
 }
 
 }  // namespace
@@ -989,7 +996,8 @@ cudaError_t launch_select_compact(const Problem& p, const float* scores, const f
                                   const int32_t* budgets, const uint8_t* modality,
                                   int64_t* offsets, int32_t* idx, const uint16_t* k,
                                   const uint16_t* v, uint16_t* k_out, uint16_t* v_out,
-                                  long long capacity_rows, uint32_t* status, cudaStream_t stream) {
+                                  long long capacity_rows, uint32_t* status, cudaStream_t stream,
+                                  bool after_score) {
     if (general_select(p)) {
         if (select_general_smem(p, true) > kFusedSmemLimit) {
             cudaError_t e = launch_select_cap(p, scores, text_scores, budgets, modality, offsets,
@@ -1008,9 +1016,9 @@ cudaError_t launch_select_compact(const Problem& p, const float* scores, const f
     if (const int nw = warp_select_warps(p)) {
         if (p.d == 64)
             return launch_sel_warp<8>(p, nw, scores, budgets, modality, offsets, idx, k, v, k_out,
-                                      v_out, capacity_rows, status, stream);
+                                      v_out, capacity_rows, status, stream, after_score);
         return launch_sel_warp<16>(p, nw, scores, budgets, modality, offsets, idx, k, v, k_out,
-                                   v_out, capacity_rows, status, stream);
+                                   v_out, capacity_rows, status, stream, after_score);
     }
     if (select_smem(p, true) > kFusedSmemLimit) {
         cudaError_t e = launch_select_cap(p, scores, nullptr, budgets, modality, offsets, idx,
@@ -1021,9 +1029,9 @@ cudaError_t launch_select_compact(const Problem& p, const float* scores, const f
     }
     if (p.d == 64)
         return launch_sel<true, 8>(p, scores, budgets, modality, offsets, idx, k, v, k_out, v_out,
-                                   capacity_rows, status, stream);
+                                   capacity_rows, status, stream, after_score);
     return launch_sel<true, 16>(p, scores, budgets, modality, offsets, idx, k, v, k_out, v_out,
-                                capacity_rows, status, stream);
+                                capacity_rows, status, stream, after_score);
 }
 
 }  // namespace tgvkv
