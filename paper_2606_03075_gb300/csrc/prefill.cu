@@ -715,6 +715,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                         }
                     }
                 }
+                __syncwarp();   // (the vote orders no memory: see the pairs' wait_all)
                 tc::fence_after_sync();
             };
             // the next tile to take QK of: tile j of item n (hi < 0: no more)
@@ -827,6 +828,9 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                     }
                 }
                 if (mine && lane >= 2) my_phase ^= 1u;
+                // what each lane's barrier guards, for whichever lane issues the MMAs: the vote
+                // orders no memory, this does
+                __syncwarp();
                 tc::fence_after_sync();
             };
             // S = Q K^T of ring stage i; last: the tile's last use of its Q slot; alone: the
