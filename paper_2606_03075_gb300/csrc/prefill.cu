@@ -105,7 +105,7 @@ struct FSmem {
     uint64_t it_full[PIQ], it_empty[PIQ];
     // per stream; in the solo form s_full and p_full per S buffer (two tiles of the
     // stream are in flight, and a warp may be a tile ahead of another)
-    uint64_t s_full[2], p_full[2], pv_done, o_full[2], o_empty[2], turn[2], mma_done[2];
+    uint64_t s_full[2], p_full[2], o_full[2], o_empty[2], turn[2], mma_done[2];
     uint64_t l_full[2][4];              // [stream][its item % 4]
     int item_hi[PIQ], item_lhq[PIQ];
     uint32_t tmem_base;
@@ -310,7 +310,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             tc::mbar_init(&s.turn[w], 1);
             tc::mbar_init(&s.mma_done[w], 1);
         }
-        tc::mbar_init(&s.pv_done, 1);
         tc::fence_mbar_init();
     }
     if (warp == MMA_WARP) {
@@ -415,9 +414,11 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                             lsum *= alpha;
                             vsum *= alpha;
                         }
-                        // PV_{j-1} has finished: S_j came after it (solo: S_j came after
-                        // PV_{j-2}, so one of two phases is awaited)
-                        if (SOLO && j > 0 && !warp_wait_all(&s.pv_done, st & 1, abort_flag)) {
+                        // PV_{j-1} has finished: S_j came after it.  (Solo: S_j came after
+                        // PV_{j-2}; what comes after PV_{j-1} is the S of the tile after this
+                        // one, whose barrier this warp awaits for every tile, so that its phase
+                        // is known: it cannot be past that S before this warp's P.)
+                        if (SOLO && j > 0 && !warp_wait_all(&s.s_full[sb ^ 1], (st >> 1) & 1, abort_flag)) {
                             ok = false;
                             s.abort_flag = 1;
                             break;
@@ -756,10 +757,12 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 if (ok && tc::elect_one()) {
                     pv_block<D>(to, tm + (uint32_t)((g & 1) * PN), vd0 + (uint64_t)((it % PST) * SLOT),
                                 !first);
-                    tc::mma_commit(&s.pv_done);
                     if (last) tc::mma_commit(&s.o_full[1]);
                     tc::mma_commit(&s.empty[it % PST]);
-                    if (more) qk(g, it + 1);
+                    if (more)
+                        qk(g, it + 1);
+                    else    // no further tile: the softmax may still wait for PV_g here
+                        tc::mma_commit(&s.s_full[g & 1]);
                 }
                 __syncwarp();
                 if (first) ++done;

@@ -427,13 +427,17 @@ def test_evict_with_statistics_head_budgets(api, stat):
 
 # head lengths at the edges of the kernel's work split: one tile, one pair of row
 # tiles, an odd tile left over, a last tile of one row; MHA and grouped heads.
-# "few" row tiles (one per item) and "many" (pairs of them, over three per SM).
+# "few" row tiles (one per item, as always when the prompt is one tile) and "many"
+# (pairs of them, over four per SM).
 EDGES = [(1, 1, 64), (31, 4, 128), (128, 1, 128), (129, 2, 64), (256, 1, 64), (257, 3, 128),
          (385, 1, 128), (513, 2, 128)]
 
 
 def _layers(form, heads, n):
-    return 2 if form == "few" else -(-700 // (heads * -(-n // 128)))
+    tiles = heads * -(-n // 128)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    # "several" items of one tile per CTA, one after another
+    return 2 if form == "few" else 4 * sms // tiles if form == "several" else 4 * sms // tiles + 1
 
 
 @pytest.mark.parametrize("form", ["few", "many"])
@@ -478,7 +482,7 @@ def test_prefill_in_a_workspace_of_other_calls(api, L, n):
         assert api.tgvkv_status(ws) == 0
 
 
-@pytest.mark.parametrize("form", ["few", "many"])
+@pytest.mark.parametrize("form", ["few", "several", "many"])
 @pytest.mark.parametrize("first_rise", [20, 70, 140, 200, 330])
 def test_prefill_rising_logits(api, first_rise, form):
     """Logits that jump along the sequence, so that the rows' reference maximum moves
