@@ -43,8 +43,8 @@
 //   * items end for the softmax with the row sums; a further warpgroup divides O by
 //     them and stores it while the streams run the next item.
 // Measured (one launch, 28 layers of 28/4 heads, d = 128, N = 4352): 3.60 ms with
-// one tile per CTA, P in shared memory and the maximum taken for every tile, 2.53 ms
-// now (1500 TFLOP/s); 32 layers of 32 heads, N = 3008: 3.05 -> 1.68 ms, also because
+// one tile per CTA, P in shared memory and the maximum taken for every tile, 2.50 ms
+// now (1520 TFLOP/s); 32 layers of 32 heads, N = 3008: 3.05 -> 1.68 ms, also because
 // heads are worked on in batches whose K and V stay in L2.
 //
 // Solo form, for launches with few row tiles (see launch_prefill): one tile per
@@ -91,6 +91,10 @@ constexpr int P_READERS = 8 + 4 + 2, P_READERS_SOLO = 4 + 4 + 1;
 // than the block holds.
 constexpr int P_REGS = 128, SOFT_REGS = 192, OUT_REGS = 40, ROLE_REGS = 88;
 static_assert(2 * SOFT_REGS + OUT_REGS + ROLE_REGS <= 4 * P_REGS, "register split");
+// solo form: the first softmax warpgroup has no stream
+constexpr int IDLE_REGS = 24, SOLO_SOFT_REGS = 208, SOLO_OUT_REGS = 104;
+static_assert(IDLE_REGS + SOLO_SOFT_REGS + SOLO_OUT_REGS + ROLE_REGS <= 4 * P_REGS,
+              "register split, solo form");
 // TMEM columns: S_w at 128 w (P_w over its first 64), O_w from 256
 constexpr int P_TMEM_COLS = 512;
 constexpr uint32_t O_COL = 256;
@@ -185,19 +189,9 @@ __device__ __forceinline__ void mask_word(float (&x)[32], int lim) {
         if (c > lim) x[c] = -INFINITY;
 }
 
-// A row's 128 logits of a score tile (TMEM columns from ts) as 2^(x sl2 - m),
-// packed in pk in bf16 pairs; z: their fp32 sum, v: the part of it at the vision
-// keys (bits in vw, the same for every lane of the warp): whole 32-key words, or
-// MIXED, for tiles with a word of both kinds, key by key.  lim: the last visible
-// key (>= 127: all).  One branch-free block: the words' latencies overlap, and
-// warps with and without a query row run the same code.  (The mixed words' logits
-// read and exponentiated once more instead, before P is handed on: 10.77 ms for 28
-// layers of N = 8704 whose query rows stand between 32 frames, 9.75 so.)
-template <bool MIXED>
-__device__ __forceinline__ void exp_row(uint32_t ts, float sl2, float m, int lim,
-                                        const uint32_t (&vw)[4], uint32_t (&pk)[64], float& z,
-                                        float& v) {
-    float x[4][32];
+// A row's 128 logits of a score tile (TMEM columns from ts); those of keys past lim
+// (>= 127: none) become -inf.
+__device__ __forceinline__ void load_row(uint32_t ts, int lim, float (&x)[4][32]) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) tc::tmem_ld32(ts + (uint32_t)(32 * c), x[c]);
     tc::tmem_wait_ld();
@@ -205,6 +199,18 @@ __device__ __forceinline__ void exp_row(uint32_t ts, float sl2, float m, int lim
 #pragma unroll
         for (int c = 0; c < 4; ++c) mask_word(x[c], lim - 32 * c);
     }
+}
+
+// A row's 128 logits of a score tile as 2^(x sl2 - m), packed in pk in bf16 pairs; z: their fp32 sum, v: the part of it at the vision
+// keys (bits in vw, the same for every lane of the warp): whole 32-key words, or
+// MIXED, for tiles with a word of both kinds, key by key.  One branch-free block: the words' latencies overlap, and
+// warps with and without a query row run the same code.  (The mixed words' logits
+// read and exponentiated once more instead, before P is handed on: 10.77 ms for 28
+// layers of N = 8704 whose query rows stand between 32 frames, 9.75 so.)
+template <bool MIXED>
+__device__ __forceinline__ void exp_row(const float (&x)[4][32], float sl2, float m,
+                                        const uint32_t (&vw)[4], uint32_t (&pk)[64], float& z,
+                                        float& v) {
     const float2 s2 = make_float2(sl2, sl2), n2 = make_float2(-m, -m);
     z = 0.f;
     v = 0.f;
@@ -244,28 +250,17 @@ __device__ __forceinline__ float fmax3f(float a, float b, float c) {
     return r;
 }
 
-// Maximum of a row's 128 logits (keys up to lim).
-__device__ __forceinline__ float max_row(uint32_t ts, int lim) {
-    float m = -INFINITY;
-#pragma unroll 1
-    for (int w = 0; w < 4; ++w) {
-        float x[32];
-        tc::tmem_ld32(ts + (uint32_t)(32 * w), x);
-        tc::tmem_wait_ld();
-        if (!__all_sync(~0u, lim >= 127)) mask_word(x, lim - 32 * w);
-        float a = x[0], b = x[1], c = x[2], d = x[3];
+// Maximum of a row's 128 logits.
+__device__ __forceinline__ float max_row(const float (&x)[4][32]) {
+    float m[4];
 #pragma unroll
-        for (int i = 4; i < 28; i += 8) {
-            a = fmax3f(a, x[i], x[i + 1]);
-            b = fmax3f(b, x[i + 2], x[i + 3]);
-            c = fmax3f(c, x[i + 4], x[i + 5]);
-            d = fmax3f(d, x[i + 6], x[i + 7]);
-        }
-        a = fmax3f(a, x[28], x[29]);
-        b = fmax3f(b, x[30], x[31]);
-        m = fmax3f(m, fmax3f(a, b, c), d);
+    for (int w = 0; w < 4; ++w) {
+        m[w] = x[w][0];
+#pragma unroll
+        for (int i = 1; i < 31; i += 2) m[w] = fmax3f(m[w], x[w][i], x[w][i + 1]);
+        m[w] = fmaxf(m[w], x[w][31]);
     }
-    return m;
+    return fmaxf(fmax3f(m[0], m[1], m[2]), m[3]);
 }
 
 template <int D, bool SOLO>
@@ -341,10 +336,14 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         return it;
     };
 
-    if (warp < OUT_WARP) {
+    // the softmax warps wait for the output warps' tables
+    constexpr int TABLE_READERS = SOLO ? 8 * 32 : 12 * 32;
+    if (SOLO && warp < 4) {
+        tc::regs_dec<IDLE_REGS>();
+    } else if (warp < OUT_WARP) {
         // -------------------------------------------------------- softmax
-        tc::regs_inc<SOFT_REGS>();
-        tc::named_bar_sync(2, LOAD_WARP * 32);   // the output warps' tables
+        tc::regs_inc<SOLO ? SOLO_SOFT_REGS : SOFT_REGS>();
+        tc::named_bar_sync(2, TABLE_READERS);
         const int w = warp >> 2, quarter = warp & 3;         // stream, lane quarter
         const int r = quarter * 32 + lane;                   // this thread's row = TMEM lane
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -352,7 +351,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         const float sl2 = p.scale_log2;
         int st = 0, items = 0;        // tiles and items of this stream so far
         bool ok = true;
-        for (int n = 0; ok && !(SOLO && w == 0); ++n) {
+        for (int n = 0; ok; ++n) {
             const PItem itm = warp_item(n);
             if (itm.hi < 0) break;
             const int t = itm.hi - 1 + w;
@@ -400,13 +399,17 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 float z, v;
                 // With the reference the row has: a sum of at most 2^8 shows that no
                 // term is above 2^8, so that m stays.  Only otherwise (and for the
-                // first tile) is the tile's maximum looked for.
+                // first tile) is the tile's maximum looked for, in the logits that the
+                // exponentials then take.  (Read for each of the two: 3700 clocks per first
+                // tile instead of 2700; 32 layers of 32 heads of 171 tokens 56 -> 48 us, of
+                // 675 tokens 189 -> 185.)
                 bool again = j == 0;
                 for (;;) {
+                    float x[4][32];
+                    load_row(ts, lim, x);
                     if (again) {
-                        const float m_tile = max_row(ts, lim) * sl2;
+                        const float m_tile = max_row(x) * sl2;
                         const bool up = m_tile > m + kRescaleLog2;   // also the first tile
-                        if (j > 0 && !__any_sync(~0u, up)) break;
                         float alpha = 1.f;
                         if (up) {
                             alpha = fast_exp2(m - m_tile);
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                             break;
                         }
                         if (SOLO) tc::fence_after_sync();
-                        if (j > 0) {
+                        if (j > 0 && __any_sync(~0u, up)) {
 #pragma unroll 1
                             for (int c = 0; c < D / 16; ++c) {
                                 float y[16];
@@ -438,9 +441,9 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                         }
                     }
                     if (mixed)
-                        exp_row<true>(ts, sl2, m, lim, vw, pk, z, v);
+                        exp_row<true>(x, sl2, m, vw, pk, z, v);
                     else
-                        exp_row<false>(ts, sl2, m, lim, vw, pk, z, v);
+                        exp_row<false>(x, sl2, m, vw, pk, z, v);
                     if (again || __all_sync(~0u, z <= kTermLimit)) break;
                     again = true;
                 }
@@ -474,7 +477,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         if (!ok) raise_status(status, TGVKV_STATUS_TIMEOUT);
     } else if (warp < LOAD_WARP) {
         // -------------------------------------------------------- output rows
-        tc::regs_dec<OUT_REGS>();
+        tc::regs_dec<SOLO ? SOLO_OUT_REGS : OUT_REGS>();
         // The tables: the query rows of each row tile t, indices wtile[t] ..
         // wtile[t + 1] of text_pos (positions ascend), as the first row at or after
         // position 128 t; their positions as bits; and the modality as bits, whole
@@ -507,7 +510,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                 if (lane == 0 && w0 + i * WARPS < 4 * n_qt) s.vis[w0 + i * WARPS] = bits;
             }
         }
-        tc::named_bar_sync(2, LOAD_WARP * 32);
+        tc::named_bar_sync(2, TABLE_READERS);
         const int quarter = warp & 3;
         const int r = quarter * 32 + lane;
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -517,6 +520,21 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         for (int n = 0; ok; ++n) {
             const PItem itm = warp_item(n);
             if (itm.hi < 0) break;
+            // q_text[l][h][r] = q[l][h][text_pos[r]] for the query rows of the item's
+            // tiles, 16 bytes a lane, while the softmax works on them (after the output, the
+            // last item's copy ended the launch: 0.4 us; by a warp of its own, its code took
+            // turns with the softmax's in the instruction cache, 32 layers of 32 heads of 384
+            // tokens 82 -> 90 us)
+            const int ws = s.wtile[itm.hi > 0 && !SOLO ? itm.hi - 1 : itm.hi], we = s.wtile[itm.hi + 1];
+            const uint16_t* qh = q + (size_t)itm.lhq * p.N * D;
+            uint16_t* qt = q_text + (size_t)itm.lhq * p.n_win * D;
+#pragma unroll 4
+            for (int e = ws + ow * RPI + lane / LPR; e < we; e += WARPS * RPI) {
+                const int pos = __ldg(text_pos + e);
+                if (pos < 0 || pos >= p.N) continue;
+                reinterpret_cast<uint4*>(qt + (size_t)e * D)[lane % LPR] =
+                    __ldg(reinterpret_cast<const uint4*>(qh + (size_t)pos * D) + lane % LPR);
+            }
             for (int w = SOLO ? 1 : 0; ok && w < 2; ++w) {
                 const int t = itm.hi - 1 + w;
                 if (t < 0) continue;
@@ -556,18 +574,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                         }
                     }
                 }
-            }
-            // q_text[l][h][r] = q[l][h][text_pos[r]] for the query rows of the item's
-            // tiles, 16 bytes a lane
-            const int ws = s.wtile[itm.hi > 0 && !SOLO ? itm.hi - 1 : itm.hi], we = s.wtile[itm.hi + 1];
-            const uint16_t* qh = q + (size_t)itm.lhq * p.N * D;
-            uint16_t* qt = q_text + (size_t)itm.lhq * p.n_win * D;
-#pragma unroll 4
-            for (int e = ws + ow * RPI + lane / LPR; e < we; e += WARPS * RPI) {
-                const int pos = __ldg(text_pos + e);
-                if (pos < 0 || pos >= p.N) continue;
-                reinterpret_cast<uint4*>(qt + (size_t)e * D)[lane % LPR] =
-                    __ldg(reinterpret_cast<const uint4*>(qh + (size_t)pos * D) + lane % LPR);
             }
         }
         if (!ok) raise_status(status, TGVKV_STATUS_TIMEOUT);
