@@ -38,8 +38,8 @@
 //     tile's maximum is known: a sum of at most 2^8 shows that no term is above
 //     2^8, so the reference stays; the maximum is looked for only otherwise;
 //   * the row's 128 terms are one branch-free block without spills (192 registers
-//     by setmaxnreg), and what is rare is rolled: straight-line code that is cold
-//     costs about 20 clocks per instruction;
+//     by setmaxnreg), the same for all four warps of a tile, and what is rare is
+//     rolled: straight-line code that is cold costs about 20 clocks per instruction;
 //   * items end for the softmax with the row sums; a further warpgroup divides O by
 //     them and stores it while the streams run the next item.
 // Measured (one launch, 28 layers of 28/4 heads, d = 128, N = 4352): 3.60 ms with
@@ -204,7 +204,7 @@ __device__ __forceinline__ void load_row(uint32_t ts, int lim, float (&x)[4][32]
 // A row's 128 logits of a score tile as 2^(x sl2 - m), packed in pk in bf16 pairs; z: their fp32 sum, v: the part of it at the vision
 // keys (bits in vw, the same for every lane of the warp): whole 32-key words, or
 // MIXED, for tiles with a word of both kinds, key by key.  One branch-free block: the words' latencies overlap, and
-// warps with and without a query row run the same code.  (The mixed words' logits
+// rows with and without a query run the same code.  (The mixed words' logits
 // read and exponentiated once more instead, before P is handed on: 10.77 ms for 28
 // layers of N = 8704 whose query rows stand between 32 frames, 9.75 so.)
 template <bool MIXED>
@@ -362,8 +362,14 @@ __global__ void __launch_bounds__(P_THREADS, 1)
             // plus those at the tile's positions before (rows out of order, which the
             // status reports, may count past the end)
             int wi = -1;
+            bool want_v = false;
             if (p.n_win > 0) {
                 const uint4 u = *reinterpret_cast<const uint4*>(&s.rows[4 * t]);
+                // for the whole tile, so that its four warps run the same code: with only the
+                // warps that hold a query row in the mixed form the two forms took turns in the
+                // instruction cache (32 layers of 32 heads of 100 tokens 30.1 -> 25.7 us, of 171
+                // tokens 47.5 -> 45.3)
+                want_v = (u.x | u.y | u.z | u.w) != 0u;
                 const uint32_t own = quarter == 0 ? u.x : quarter == 1 ? u.y : quarter == 2 ? u.z : u.w;
                 if ((own >> lane) & 1u) {
                     wi = s.wtile[t] + __popc(own & ((1u << lane) - 1u)) + (quarter > 0 ? __popc(u.x) : 0) +
@@ -371,7 +377,6 @@ __global__ void __launch_bounds__(P_THREADS, 1)
                     if (!valid || wi >= p.n_win) wi = -1;
                 }
             }
-            const bool want_v = __any_sync(~0u, wi >= 0);
             float m = -INFINITY, lsum = 0.f, vsum = 0.f;
             for (int j = 0; j <= t; ++j) {
                 uint32_t vw[4] = {0u, 0u, 0u, 0u};
