@@ -977,14 +977,21 @@ cudaError_t launch_prefill(const Problem& p, const uint16_t* q, const uint16_t* 
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + lay.status);
     const int sms = device_sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;
-    // Up to four row tiles per SM the pairs leave SMs idle or end unevenly, and a
-    // pair's step is no shorter for having the SM's neighbours idle: one head pair of
-    // 8000 keys 68 us solo, 111 us in pairs (d = 128), 14 heads of 2833 keys 46 / 51,
-    // 32 heads of 858 keys 25 / 30, 28 heads of 2500 keys (3.7 tiles per SM, d = 64) 41 /
-    // 47; above, the pairs' shared K and V tiles win (56 heads of 1685 keys, 5 tiles per
-    // SM: 142 / 120 us).  One tile per head makes no pair: 1024 heads of 100 keys 35 / 39.
+    // One tile per item, or two.  Mean time of the one-tile form over that of the pairs,
+    // for heads of 100 to 3200 keys, d = 64 and 128, 1 to 100 layers of 8 and 28 heads, by
+    // row tiles per SM and (across) row tiles per head:
+    //                1     2     3     4     5    >5
+    //     up to 1  1.00  0.94  0.90  0.88  0.83  0.80   a pair's tiles wait in one SM
+    //         1-2  1.02  1.15  1.03  1.04  0.96  0.94
+    //         2-3  0.99  1.00  1.04  0.98  0.93  0.96
+    //         3-4  0.97  1.06  0.92  1.10  1.04  0.98
+    //     above 4  0.98  0.99  0.97  0.99  1.13  1.11   the pairs share K and V tiles
+    // (between, the two round up to whole items per SM at different sizes).  So: one-tile
+    // heads, which make no pair, and launches of up to a tile per SM take the one-tile form;
+    // two-tile heads pairs; longer ones the one-tile form up to four tiles per SM.
     const int n_qt = (p.N + PM - 1) / PM;
-    const bool solo = n_qt == 1 || (long long)p.L * p.H_q * n_qt <= 4ll * sms;
+    const long long tiles = (long long)p.L * p.H_q * n_qt;
+    const bool solo = n_qt == 1 || tiles <= sms || (n_qt > 2 && tiles <= 4ll * sms);
     const auto launch = p.d == 64 ? (solo ? launch_prefill_d<64, true> : launch_prefill_d<64, false>)
                                   : (solo ? launch_prefill_d<128, true> : launch_prefill_d<128, false>);
     return launch(p, q, k, v, modality, text_pos, o, q_text, row_stats, work_counter, status, sms,
