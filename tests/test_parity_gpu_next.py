@@ -388,9 +388,11 @@ def test_decode_full_size(api, name):
     P.assert_close(of, reff, "decode, full cache", floor=DEC_FLOOR)
 
 
-def test_decode_empty_sets_give_zero(api):
-    """No text token and a zero budget: every set is empty and the output is 0."""
-    wl = synth.custom("all_vision", 2, 4, 2, 64, [("vision", 70)], window="all_text",
+@pytest.mark.parametrize("L", [2, 90])
+def test_decode_empty_sets_give_zero(api, L):
+    """No text token and a zero budget: every set is empty and the output is 0 (few
+    sets and many: the two forms of the merge)."""
+    wl = synth.custom("all_vision", L, 4, 2, 64, [("vision", 70)], window="all_text",
                       ratios=(0.0,))
     desc = api.desc_for_workload(wl)
     offsets = torch.zeros(wl.L * wl.H_kv + 1, dtype=torch.int64, device="cuda")
@@ -399,15 +401,28 @@ def test_decode_empty_sets_give_zero(api):
     assert np.array_equal(o, np.zeros_like(o))
 
 
+# Steps in a row: few short sets; many heads per group; few sets split over hundreds of
+# streams each (whose merge takes as long as the row streams); sets enough for the merge
+# by one warp.
+STEP_CASES = dict(
+    tiny=DECODE_CASES["tiny"], wide_group=DECODE_CASES["wide_group"],
+    long_sets=synth.custom("long_sets", 1, 28, 4, 128, [("text", 32), ("vision", 6000), ("text", 60)],
+                           ratios=(0.9,)),
+    many_sets=synth.custom("many_sets", 20, 16, 8, 64, [("text", 9), ("vision", 300), ("text", 9)],
+                           ratios=(0.5,)))
+
+
 @pytest.mark.parametrize("captured", [False, True])
-@pytest.mark.parametrize("name", ["tiny", "wide_group"])
+@pytest.mark.parametrize("name", sorted(STEP_CASES))
 def test_decode_steps_back_to_back(api, name, captured):
     """A decode step may be launched while the kernel before it still runs.  Steps in
-    one workspace and one set of buffers -- each after an eviction that rewrites the
-    rows and the offsets, and after a copy that rewrites the queries, or straight
-    after another step -- give the same bits without a wait between them as with one,
-    also replayed from a graph."""
-    wl = DECODE_CASES[name]
+    one workspace -- after an eviction that rewrites the rows and the offsets, after a
+    copy that rewrites the queries, and several straight after one another, each with
+    queries of its own and over the compacted and the full cache in turn, so that every
+    step's partial results differ from those the step before left in their place --
+    give the same bits without a wait between them as with one, also replayed from a
+    graph."""
+    wl = STEP_CASES[name]
     desc = api.desc_for_workload(wl)
     ws = api.new_workspace(desc)
     devs = [P.device_inputs(synth.generate(wl, seed=s)) for s in (6, 7)]
@@ -415,19 +430,26 @@ def test_decode_steps_back_to_back(api, name, captured):
     out = api.alloc_outputs(desc, max(ratios))
     qs = [torch.from_numpy(_decode_q(wl, s)).cuda().view(torch.bfloat16) for s in (1, 2, 3)]
     q = torch.empty_like(qs[0])
-    shape = (6, wl.L, wl.H_q, wl.d)
+    whole = torch.arange(wl.L * wl.H_kv + 1, dtype=torch.int64, device="cuda") * wl.N
+    shape = (16, wl.L, wl.H_q, wl.d)
 
     def steps(o, wait):
-        for i in range(6):
-            if i % 3 == 0:
-                dev, ratio = devs[i // 3], ratios[i // 3]
+        for i in range(16):
+            dev, ratio = devs[i // 8], ratios[i // 8]
+            if i % 8 == 0:
                 api.tgvkv_evict(desc, dev["q"], dev["k"], dev["v"], dev["modality"],
                                 dev["text_pos"], dev["w"], ratio, out, ws)
                 wait()
-            if i % 3 != 2:
-                q.copy_(qs[i % 3])
+            if i % 8 == 1:
+                q.copy_(qs[1])
                 wait()
-            api.tgvkv_decode(desc, q, out.k_out, out.v_out, out.offsets, o[i], ws)
+            qi = q if i % 8 == 1 else qs[i % 3]
+            if i % 8 < 5:      # one cache, other queries each step
+                api.tgvkv_decode(desc, qi, out.k_out, out.v_out, out.offsets, o[i], ws)
+            else:              # the caches in turn: other splits too
+                k, v, off = ((dev["k"].view(-1, wl.d), dev["v"].view(-1, wl.d), whole) if i % 2
+                             else (out.k_out, out.v_out, out.offsets))
+                api.tgvkv_decode(desc, qi, k, v, off, o[i], ws)
             wait()
 
     ref = torch.full(shape, float("nan"), device="cuda")
@@ -472,14 +494,28 @@ def _ragged_decode(api, L, H_kv, G, d, lens, base, spare, seed):
     return o, ref
 
 
+@pytest.mark.parametrize("L", [3, 30])
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("G", [1, 4, 12])
-def test_decode_ragged_csr(api, d, G):
-    """Decode over ragged CSR layouts, element by element against the oracle."""
-    L, H_kv = 3, 6
-    lens = _RAGGED_LENS
+def test_decode_ragged_csr(api, d, G, L):
+    """Decode over ragged CSR layouts, element by element against the oracle (18 sets,
+    merged by sixteen warps each, and 180, by one)."""
+    H_kv = 6
+    lens = _RAGGED_LENS * (L // 3)
     o, ref = _ragged_decode(api, L, H_kv, G, d, lens, base=5, spare=37, seed=20 + G + d)
     P.assert_close(o, ref, f"decode, ragged CSR (G={G}, d={d})", floor=DEC_FLOOR)
+
+
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("G,d", [(1, 64), (7, 128)])
+def test_decode_at_the_line_between_the_merges(api, G, d, over):
+    """The most sets that sixteen warps merge each (eight streams per SM, sixteen streams
+    per set), and one set more."""
+    sets = torch.cuda.get_device_properties(0).multi_processor_count * 8 // 16 + over
+    rng = np.random.default_rng(60 + over)
+    lens = rng.integers(0, 200, sets).tolist()
+    o, ref = _ragged_decode(api, sets, 1, G, d, lens, base=3, spare=9, seed=40 + G)
+    P.assert_close(o, ref, f"decode, {sets} sets (G={G}, d={d})", floor=DEC_FLOOR)
 
 
 @pytest.mark.parametrize("G", [1, 7])
@@ -490,13 +526,15 @@ def test_decode_one_long_set(api, G):
     P.assert_close(o, ref, f"decode, one long set (G={G})", floor=DEC_FLOOR)
 
 
-def test_decode_csr_past_capacity(api):
+@pytest.mark.parametrize("L", [1, 90])
+def test_decode_csr_past_capacity(api, L):
     """A CSR whose last set runs past the rows the buffers hold: the kernel
-    reads no row from capacity_rows on and reports TGVKV_STATUS_INDEX."""
-    wl = synth.custom("short_cache", 1, 4, 2, 128, [("text", 8), ("vision", 300), ("text", 8)])
+    reads no row from capacity_rows on and reports TGVKV_STATUS_INDEX (both forms of
+    the merge, which does the check)."""
+    wl = synth.custom("short_cache", L, 4, 2, 128, [("text", 8), ("vision", 300), ("text", 8)])
     desc = api.desc_for_workload(wl)
     rows = torch.zeros((100, wl.d), dtype=torch.bfloat16, device="cuda")
-    offsets = torch.tensor([0, 60, 180], dtype=torch.int64, device="cuda")
+    offsets = torch.tensor([0] + [60] * (2 * L - 1) + [180], dtype=torch.int64, device="cuda")
     ws = api.new_workspace(desc)
     out = torch.empty((desc.L, desc.H_q, desc.d), dtype=torch.float32, device="cuda")
     qd = torch.from_numpy(_decode_q(wl, 3)).cuda().view(torch.bfloat16)
@@ -618,11 +656,13 @@ def test_widened_paths_back_to_back_stay_clean(api):
                 else:
                     np.testing.assert_array_equal(snap[0], first[0])
                     np.testing.assert_array_equal(snap[1], first[1])
-        qd = torch.from_numpy(_decode_q(wl, 14)).cuda().view(torch.bfloat16)
-        o1 = torch.empty((wl.L, wl.H_q, wl.d), dtype=torch.float32, device="cuda")
-        o2 = torch.empty_like(o1)
-        api.tgvkv_decode(desc, qd, out.k_out, out.v_out, out.offsets, o1, ws)
-        for _ in range(20):
-            api.tgvkv_decode(desc, qd, out.k_out, out.v_out, out.offsets, o2, ws)
+        # two queries in turn, so that a step's partial results are not the last one's
+        qd = [torch.from_numpy(_decode_q(wl, s)).cuda().view(torch.bfloat16) for s in (14, 15)]
+        o = torch.empty((22, wl.L, wl.H_q, wl.d), dtype=torch.float32, device="cuda")
+        for i in range(22):
+            api.tgvkv_decode(desc, qd[i % 2], out.k_out, out.v_out, out.offsets, o[i], ws)
+            if i < 2:
+                torch.cuda.synchronize()
         assert api.tgvkv_status(ws) == 0
-        assert torch.equal(o1, o2)
+        for i in range(2, 22):
+            assert torch.equal(o[i], o[i % 2])
