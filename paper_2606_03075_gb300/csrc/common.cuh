@@ -128,6 +128,26 @@ __device__ __forceinline__ float fast_log2(float x) {
     return y;
 }
 
+// Three-input maximum (PTX max.f32 with three sources).
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+__device__ __forceinline__ float max32(const float (&x)[32]) {
+    float a = fmax3(x[0], x[1], x[2]), b = fmax3(x[3], x[4], x[5]), c = fmax3(x[6], x[7], x[8]);
+    float d = fmax3(x[9], x[10], x[11]), e = fmax3(x[12], x[13], x[14]);
+    float f = fmax3(x[15], x[16], x[17]), g = fmax3(x[18], x[19], x[20]);
+    float h = fmax3(x[21], x[22], x[23]), i = fmax3(x[24], x[25], x[26]);
+    float j = fmax3(x[27], x[28], x[29]), k = fmaxf(x[30], x[31]);
+    a = fmax3(a, b, c);
+    d = fmax3(d, e, f);
+    g = fmax3(g, h, i);
+    j = fmaxf(j, k);
+    return fmaxf(fmax3(a, d, g), j);
+}
+
 // Packed pairs of fp32 (Blackwell f32x2 FMA-pipe instructions).
 union F2 {
     float2 f;

@@ -243,24 +243,9 @@ __device__ __forceinline__ void exp_row(const float (&x)[4][32], float sl2, floa
     }
 }
 
-// Three-input maximum (PTX max.f32 with three sources).
-__device__ __forceinline__ float fmax3f(float a, float b, float c) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-
 // Maximum of a row's 128 logits.
 __device__ __forceinline__ float max_row(const float (&x)[4][32]) {
-    float m[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        m[w] = x[w][0];
-#pragma unroll
-        for (int i = 1; i < 31; i += 2) m[w] = fmax3f(m[w], x[w][i], x[w][i + 1]);
-        m[w] = fmaxf(m[w], x[w][31]);
-    }
-    return fmaxf(fmax3f(m[0], m[1], m[2]), m[3]);
+    return fmaxf(fmax3(max32(x[0]), max32(x[1]), max32(x[2])), max32(x[3]));
 }
 
 template <int D, bool SOLO>

@@ -959,7 +959,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         s.abort_flag = 1;
                     }
                     if (ok) tc::fence_after_sync();
-                    int blk, ktile, ccol, rcol, rs, nch, rpg, minp;
+                    int blk, ktile, ccol, rcol, rs, nch, rpg;
                     bool act;
                     if (mode == MODE_PAIR) {
                         blk = 0;
@@ -970,7 +970,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         rcol = 64 * (wi & 1);
                         nch = 2;
                         rpg = rpgB;
-                        minp = Item::pick(itm.minp, rs);
                     } else if (mode == MODE_SINGLE) {
                         blk = wi >> 1;
                         ktile = Item::pick(kt, blk);
@@ -980,7 +979,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         rcol = 64 * (wi & 1);
                         nch = 2;
                         rpg = itm.rpg[0];
-                        minp = itm.minp[0];
                     } else {
                         blk = wi >> 1;
                         ktile = Item::pick(kt, blk);
@@ -990,7 +988,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         ccol = 128 * blk + rcol;
                         nch = 1;
                         rpg = itm.rpg[0];
-                        minp = itm.minp[0];
                     }
                     float sum = 0.f;
                     if (!ok) {
@@ -1023,13 +1020,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                             sum = (a.x + a.y) + (c.x + c.y);
                         } else {
                             for (int ch = 0; ch < nch; ++ch) {
-                                bool all_vis = last <= minp;
+                                bool all_vis = last <= itm.minp[0];
                                 if (mode == MODE_PAIR) {
                                     const int grp = (rcol >> 5) + ch;
                                     // no row of the group sees these keys (a tile of rows that
-                                // stand far apart: 28 layers, 1920 rows between 32 frames,
-                                // 1491 -> 1455 us)
-                                if (ktile * BN > s.grp_max[rs][grp]) {
+                                    // stand far apart: 28 layers, 1920 rows between 32 frames,
+                                    // 1491 -> 1455 us)
+                                    if (ktile * BN > s.grp_max[rs][grp]) {
                                         if (ch == nch - 1) release_acc(&s.s_empty[b], lane);
                                         continue;
                                     }
@@ -1054,9 +1051,8 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                         const uint32_t word = s.vmask[ktile][quarter];
                         if ((word >> lane) & 1u) {
                             const int vr = s.vq[ktile][quarter] + __popc(word & lt_mask);
-                            float* out = mode == MODE_PAIR
-                                             ? score_part + ((size_t)itm.lh[0] * p.T + 2 * itm.pidx + rs) * p.N_v
-                                             : scores + (size_t)Item::pick(itm.lh, mode == MODE_PACKED ? blk : 0) * p.N_v;
+                            float* out =
+                                scores + (size_t)Item::pick(itm.lh, mode == MODE_PACKED ? blk : 0) * p.N_v;
                             if (vr < p.N_v) atomicAdd(out + vr, sum);
                         }
                     }
