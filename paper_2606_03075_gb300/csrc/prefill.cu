@@ -329,7 +329,9 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         // -------------------------------------------------------- softmax
         tc::regs_inc<SOLO ? SOLO_SOFT_REGS : SOFT_REGS>();
         tc::named_bar_sync(2, TABLE_READERS);
-        const int w = warp >> 2, quarter = warp & 3;         // stream, lane quarter
+        // Stream and row tile come from lane 0, so that the branches on them are seen to be
+        // the warp's (64-dim heads, 8 of 2511 keys 22.8 -> 22.0 us, 96 of 2286 82.2 -> 78.8).
+        const int w = __shfl_sync(~0u, warp >> 2, 0), quarter = warp & 3;   // stream, lane quarter
         const int r = quarter * 32 + lane;                   // this thread's row = TMEM lane
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
         const uint32_t to = tl + O_COL + (uint32_t)(w * D);
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(P_THREADS, 1)
         for (int n = 0; ok; ++n) {
             const PItem itm = warp_item(n);
             if (itm.hi < 0) break;
-            const int t = itm.hi - 1 + w;
+            const int t = __shfl_sync(~0u, itm.hi, 0) - 1 + w;
             if (t < 0) continue;
             const int pos = t * PM + r;
             const bool valid = pos < p.N;
