@@ -100,7 +100,11 @@ constexpr int P_TMEM_COLS = 512;
 constexpr uint32_t O_COL = 256;
 constexpr float kRescaleLog2 = 8.f;     // a stale reference maximum may trail by 2^8
 constexpr float kTermLimit = 256.f;      // 2^kRescaleLog2
-constexpr size_t kBatchBytes = 48u << 20;   // K and V of the heads worked on together
+// K and V of the heads worked on together, so that they stay in L2: 12 to 64 MB take the
+// same time within 1.5%; one group at a time 179 us for 32 layers of 32 heads of 675
+// tokens (167 so), 96 MB 1789 us for 3008 tokens (1727), all heads 1976, and 28 layers of
+// 28/4 heads of 8704 tokens 9.66 ms (9.26).
+constexpr size_t kBatchBytes = 48u << 20;
 
 template <int D>
 struct FSmem {
