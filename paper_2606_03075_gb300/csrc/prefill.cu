@@ -43,8 +43,8 @@
 //   * items end for the softmax with the row sums; a further warpgroup divides O by
 //     them and stores it while the streams run the next item.
 // Measured (one launch, 28 layers of 28/4 heads, d = 128, N = 4352): 3.60 ms with
-// one tile per CTA, P in shared memory and the maximum taken for every tile, 2.50 ms
-// now (1520 TFLOP/s); 32 layers of 32 heads, N = 3008: 3.05 -> 1.68 ms, also because
+// one tile per CTA, P in shared memory and the maximum taken for every tile, 2.46 ms
+// now (1550 TFLOP/s); 32 layers of 32 heads, N = 3008: 3.05 -> 1.68 ms, also because
 // heads are worked on in batches whose K and V stay in L2.
 //
 // Solo form, for launches with few row tiles (see launch_prefill): one tile per
