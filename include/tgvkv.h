@@ -22,7 +22,8 @@
  * - Every call is asynchronous on `stream` (a cudaStream_t passed as void*;
  *   NULL = the legacy default stream).  Some kernels are programmatic
  *   dependents: they may be scheduled while the kernel before them ends, a
- *   caller's too, and wait for it on the device before they touch any buffer.
+ *   caller's too, and wait for it on the device; no buffer is touched before
+ *   the caller's kernels ahead of the call have finished.
  * - Arguments are validated on the host before any launch; a bad argument
  *   returns TGVKV_ERR_INVALID_ARG / TGVKV_ERR_UNSUPPORTED and launches nothing.
  *   Data-dependent faults found on the device (a query position out of range,

@@ -358,10 +358,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         tc::mbar_init(&s.mma_done, 2);
         tc::fence_mbar_init();
     }
-    if (warp == 1) {
-        tc::tmem_alloc(&s.tmem_base, TMEM_COLS);
-        tc::tmem_relinquish();
-    }
     if (tid == NTHREADS - 1) {
         tc::tma_prefetch_desc(&tmap_q);
         tc::tma_prefetch_desc(&tmap_k);
@@ -375,6 +371,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     // 112 tokens, 86.4 / 90.0 for 1024 heads of 675, 366 / 370 for 1024 heads of 3008; the
     // first loads ahead of the tables: no difference.)
     griddep_wait();
+    // (The tensor memory too is taken only now: a kernel before this one that signals
+    // first and allocates its own later would otherwise wait for this CTA, which waits for it.)
+    if (warp == 1) {
+        tc::tmem_alloc(&s.tmem_base, TMEM_COLS);
+        tc::tmem_relinquish();
+    }
     if (blockIdx.x == 0) {
         for (int i = tid; i < p.n_win; i += NTHREADS) {
             const int pi = __ldcg(text_pos + i);
